@@ -425,9 +425,11 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
             }
             if (!decided && previous_left_nothing(pub_w, p.cp.step_id, decided)) {
               // Stop at this K block: the hidden stage is completed empty and
-              // carries the stop mark to the MMA warp, which has consumed
-              // every W stage issued so far by the time it sees it.
-              *sm.skip = 1;
+              // carries the stop mark, the K block's number (a single-kernel
+              // step is one chunk), to the MMA warp, which consumes every
+              // stage issued before it first: no copy may be in flight when
+              // the CTA leaves or its shared memory is used for the commit.
+              *sm.skip = g * KB + kb + 1;
               mbar_arrive(&sm.full_b[rb.slot]);
               skipped = true;
               break;
@@ -505,7 +507,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
               ok = false;
               break;
             }
-            if (spec && *sm.skip) {
+            if (spec && *sm.skip == g * KB + kb + 1) {
               skipped = true;
               break;
             }
@@ -598,8 +600,9 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
             ok = false;
             break;
           }
-          if (spec && *sm.skip) {
-            ok = false;  // stop: nothing of this step is written
+          const int stop = spec ? *sm.skip : 0;
+          if (stop > g * KB && stop <= (g + 1) * KB) {
+            ok = false;  // stopped in this group: nothing of this step is written
             break;
           }
           tc_fence_after();
@@ -643,8 +646,9 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
             ok = false;
             break;
           }
-          if (spec && *sm.skip) {
-            ok = false;  // stop: nothing of this step is written
+          const int stop = spec ? *sm.skip : 0;
+          if (stop > g * KB && stop <= (g + 1) * KB) {
+            ok = false;  // stopped in this group: nothing of this step is written
             break;
           }
           tc_fence_after();

@@ -258,10 +258,11 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
             break;
           }
           if (!decided && previous_left_nothing(pub_w, p.cp.step_id, decided)) {
-            // Stop: the rows stage completes empty and carries the stop mark
-            // to the MMA thread, which has consumed every W stage issued so
-            // far by the time it sees it.
-            *sm.skip = 1;
+            // Stop: the rows stage completes empty and carries the stop mark,
+            // this K block's number, to the MMA thread, which consumes every
+            // stage issued before it first (no copy may be in flight when the
+            // CTA leaves or its shared memory is used for the commit).
+            *sm.skip = g * KB + kb + 1;
             mbar_arrive(&sm.full_h[rh.slot]);
             g = pl.n_groups;
             break;
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
             ok = false;
             break;
           }
-          if (spec && *sm.skip) {
+          if (spec && *sm.skip == g * KB + kb + 1) {
             skipped = true;
             break;
           }
@@ -385,8 +386,9 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
         ok = false;
         break;
       }
-      if (spec && *sm.skip) {
-        ok = false;  // stop: nothing of this step is written
+      const int stop = spec ? *sm.skip : 0;
+      if (stop > g * KB && stop <= (g + 1) * KB) {
+        ok = false;  // stopped in this group: nothing of this step is written
         break;
       }
       tc_fence_after();
