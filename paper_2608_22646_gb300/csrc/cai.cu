@@ -261,6 +261,8 @@ struct cai_ctx {
   bool stage_by_word = false;
   bool fused = false;    // single-kernel step (B P <= 64)
   bool rows_head = false;  // the single-kernel step runs lm_head_rows_kernel
+  int step_box = kBoxRowsB;  // rows per TMA box of a single-kernel step's rows: the rows-operand
+                             // head loads a K block of them as one box (each copy costs its issue)
   // Vocabulary shard (cai_init_vocab_shard): the context's LM head covers the
   // rows [v_off, v_off + cfg.V) of a vocabulary of V_total rows; a step is
   // cai_shard_head, an exchange of every shard's triples, cai_shard_commit.
@@ -602,7 +604,7 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
   } else {
     if (stage_slot < 0 && hid != c->hid_mapped) {
       // The single-kernel step reads the caller's [B P, H] rows through TMA.
-      if (!make_map(&c->tm_hid, hid, c->BP, cfg.H, kBoxRowsB)) return CAI_ERR_ARG;
+      if (!make_map(&c->tm_hid, hid, c->BP, cfg.H, c->step_box)) return CAI_ERR_ARG;
       c->hid_mapped = hid;
     }
     // With the final norm the LM-head kernel computes the row scales from
@@ -851,6 +853,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   const char* rh_env = std::getenv("CAI_ROWS_HEAD");
   if (c->fused && c->BP <= kRowsM && !(rh_env && rh_env[0] == '0')) {
     c->rows_head = true;
+    c->step_box = c->rows_cap;
     c->head_kernel = c->norm ? lm_head_rows_kernel<true> : lm_head_rows_kernel<false>;
     cudaFuncAttributes ra{};
     if (cudaFuncGetAttributes(&ra, c->head_kernel) != cudaSuccess) {
@@ -1080,8 +1083,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     return CAI_ERR_CUDA;
   }
   if (!shard) {
-    bool ok = (!c->fused || (make_map(&c->tm_stage[0], c->stage2[0], c->BP, cfg->H, kBoxRowsB) &&
-                             make_map(&c->tm_stage[1], c->stage2[1], c->BP, cfg->H, kBoxRowsB))) &&
+    bool ok = (!c->fused || (make_map(&c->tm_stage[0], c->stage2[0], c->BP, cfg->H, c->step_box) &&
+                             make_map(&c->tm_stage[1], c->stage2[1], c->BP, cfg->H, c->step_box))) &&
               cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking) == cudaSuccess;
     for (int k = 0; ok && k < 2; ++k)
       ok = cudaEventCreateWithFlags(&c->ev_copied[k], cudaEventDisableTiming) == cudaSuccess &&

@@ -53,15 +53,26 @@
 // arms with the bytes of both.  Two accumulator buffers let the epilogue of
 // one tile overlap the next tile's MMAs.
 //
-// What bounds a step: reading W from HBM with one row tile; with two or more,
-// the MMAs.  The tensor core runs the MMAs of the one issuing thread one after
-// another, about 63 + 0.085 N ns each (M = 256, K = 16, measured on GB300),
-// so a 160-column tile costs nearly as much per K block as a 256-column one
-// and two row tiles take twice one; each orientation issues the fewest MMAs
-// its M allows (ceil(M / 256) per vocabulary tile and K slice).  A second
-// issuing thread would run MMAs side by side, but two threads accumulating
-// into one accumulator do so in no fixed order, and the fp32 logits (and the
-// commit decisions at a threshold) would then change from run to run.
+// How stages are issued.  The producer and the MMA warp run their loops with
+// all 32 lanes, every loop bound and descriptor the same in each, and only the
+// issuing instructions are predicated on one elected lane: the descriptors and
+// coordinates then stay in uniform registers, where the TMA and MMA
+// instructions take them from.  With the loops inside `if (lane == 0)` each
+// MMA cost its thread ~50 ns and a stage 300 ns whatever its width, more than
+// its copies and its tensor work.  Measured, 4096 x 126464, one step's head:
+// M = 264 269 -> 209 us, M = 352 279 -> 238 us, M = 512 297 -> 286 us,
+// M = 2048 1.09 -> 1.04 ms, M = 128 165 -> 157 us; of it, the MMA warp alone
+// gave 42 us at M = 264 and the producer 17 us.  A wait that gives up makes its
+// lane stop waiting and issuing, not leave the loop, so that no vote is needed
+// per stage (a vote costs 1 to 4 us a step); the warp leaves together at the
+// end of the tile.
+//
+// What bounds a step: reading W from HBM with one row tile.  With two narrow
+// ones, filling the stages from L2 (26 KiB per CTA and 250 ns at N = 160, every
+// CTA at once); with wide ones the tensor cores.  A second issuing thread
+// would run MMAs side by side, but two threads accumulating into one
+// accumulator do so in no fixed order, and the fp32 logits (and the commit
+// decisions at a threshold) would then change from run to run.
 #pragma once
 
 #include <climits>
@@ -296,31 +307,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const uint32_t tmem_base = *sm.tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------ producer --
-      const uint64_t pol_a = policy_evict_last();
-      const uint32_t full0 = mapa_shared(sm.full, 0);  // the even CTA's barriers
-      PairRing r;
-      long long issued = 0;
-      bool ok = true;
-      // Swapped: a CTA's rt_rows / 2 rows (a multiple of 16) load as one box.
-      const int q1 = rt_rows / 32 - 1;
-      const int box_rows = rt_rows / 2;
-      // Bytes of one stage, both CTAs (the even CTA arms its barrier for them).
-      const uint32_t stage_tx =
-          swap ? 2u * static_cast<uint32_t>(kPairHalfBytes + box_rows * kPairBlockK * 2)
-                : 2u * kPairStageBytes;
-      for (int i = 0; i < my_tiles && ok; ++i) {
-        const int t = pair + i * n_pairs;
-        const int v = t / n_rt, j = t - v * n_rt;
-        // First row of this CTA's half of the tile's rows.
-        const int a_row = j * rt_rows + static_cast<int>(rank) * (swap ? rt_rows / 2 : kPairHalf);
-        const int w_box = (2 * v + static_cast<int>(rank)) * KB;
-        for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty)) {
-            ok = false;
-            break;
-          }
+    // -------------------------------------------------------- producer --
+    const uint64_t pol_a = policy_evict_last();
+    const uint32_t full0 = mapa_shared(sm.full, 0);  // the even CTA's barriers
+    const bool leader = elect_one();
+    PairRing r;
+    long long issued = 0;
+    bool ok = true;
+    // Swapped: a CTA's rt_rows / 2 rows (a multiple of 16) load as one box.
+    const int q1 = rt_rows / 32 - 1;
+    const int box_rows = rt_rows / 2;
+    // Bytes of one stage, both CTAs (the even CTA arms its barrier for them).
+    const uint32_t stage_tx =
+        swap ? 2u * static_cast<uint32_t>(kPairHalfBytes + box_rows * kPairBlockK * 2)
+              : 2u * kPairStageBytes;
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int t = pair + i * n_pairs;
+      const int v = t / n_rt, j = t - v * n_rt;
+      // First row of this CTA's half of the tile's rows.
+      const int a_row = j * rt_rows + static_cast<int>(rank) * (swap ? rt_rows / 2 : kPairHalf);
+      const int w_box = (2 * v + static_cast<int>(rank)) * KB;
+      for (int kb = 0; kb < KB; ++kb) {
+        ok = ok && mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
+        if (leader && ok) {
           uint8_t* dst = sm.stage + static_cast<size_t>(r.slot) * stage_stride;
           const uint32_t bar = full0 + static_cast<uint32_t>(r.slot * 8);
           // The even CTA arms the stage for the bytes of both CTAs; a copy of
@@ -334,54 +343,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             tma_load_2d_pair(dst, &tm_a, bar, kb * kPairBlockK, a_row, pol_a);
             tma_load_2d_pair_nohint(dst + kPairHalfBytes, &tm_w, bar, 0, (w_box + kb) * kPairHalf);
           }
-          ++issued;
-          r.next(n_ring);
         }
+        __syncwarp();
+        issued += ok ? 1 : 0;
+        r.next(n_ring);
       }
-      if (!ok && rank == 0) {
-        const long long f0 = issued > n_ring ? issued - n_ring : 0;
-        for (long long q = f0; q < issued; ++q)
-          pair_drain(&sm.full[q % n_ring], static_cast<uint32_t>((q / n_ring) & 1), p.err);
-      }
+      ok = __all_sync(0xffffffffu, ok);
+    }
+    if (!ok && rank == 0 && leader) {
+      const long long f0 = issued > n_ring ? issued - n_ring : 0;
+      for (long long q = f0; q < issued; ++q)
+        pair_drain(&sm.full[q % n_ring], static_cast<uint32_t>((q / n_ring) & 1), p.err);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // -------------------------------------------- MMA issuer (even CTA) --
       // Swapped: M = 256 vocabulary rows, N = the tile's rows; else M = 256
       // rows, N = 256 vocabulary rows.
       const uint32_t idesc =
           idesc_bf16_f32(256, swap ? static_cast<uint32_t>(rt_rows) : kPairTileVocab);
+      const bool leader = elect_one();
+      const uint64_t desc0 = sdesc_k_sw128(smem_addr(sm.stage));
       PairRing r;
       bool ok = true;
       for (int i = 0; i < my_tiles && ok; ++i) {
         const int acc = i & 1;
-        if (!mbar_wait_cluster(&sm.acce[acc], ((i >> 1) & 1) ^ 1u, sm.abort, p.err,
-                               kErrWaitAccEmpty)) {
-          ok = false;
-          break;
-        }
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&sm.acce[acc], ((i >> 1) & 1) ^ 1u, sm.abort,
+                                                       p.err, kErrWaitAccEmpty));
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kPairTileVocab);
         for (int kb = 0; kb < KB; ++kb) {
-          if (!mbar_wait_cluster(&sm.full[r.slot], r.phase, sm.abort, p.err, kErrWaitFull)) {
-            ok = false;
-            break;
-          }
+          ok = ok && mbar_wait_cluster(&sm.full[r.slot], r.phase, sm.abort, p.err, kErrWaitFull);
           tc_fence_after();
-          const uint32_t a_addr = smem_addr(sm.stage + static_cast<size_t>(r.slot) * stage_stride);
-          const uint32_t b_addr = a_addr + kPairHalfBytes;
+          const uint64_t a = desc0 + static_cast<uint32_t>(r.slot * stage_stride >> 4);
+          const uint64_t b = a + (kPairHalfBytes >> 4);
+          if (leader && ok) {
 #pragma unroll
-          for (int kk = 0; kk < kPairBlockK / 16; ++kk)
-            mma_bf16_pair(d_tmem, sdesc_k_sw128(a_addr + kk * 32), sdesc_k_sw128(b_addr + kk * 32),
-                          idesc, (kb | kk) != 0 ? 1u : 0u);
-          mma_commit_pair(&sm.empty[r.slot], 0x3);
+            for (int kk = 0; kk < kPairBlockK / 16; ++kk)
+              mma_bf16_pair(d_tmem, a + 2 * kk, b + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+            mma_commit_pair(&sm.empty[r.slot], 0x3);
+          }
+          __syncwarp();
           r.next(n_ring);
         }
-        if (!ok) break;
-        mma_commit_pair(&sm.accf[acc], 0x3);
+        ok = __all_sync(0xffffffffu, ok);
+        if (leader && ok) mma_commit_pair(&sm.accf[acc], 0x3);
+        __syncwarp();
       }
-      if (!ok) {
+      if (!ok && leader) {
         // Abort: wait for the MMAs already issued (they read both CTAs'
         // shared memory) before anything is released.
         mma_commit_pair(sm.drain, 0x1);

@@ -243,6 +243,17 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 
 // -------------------------------------------------------------- tcgen05 --
 
+// One lane of a converged warp (the same one at every call of the warp).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+
 // Allocate `ncols` (power of two, 32..512) columns of tensor memory; the base
 // address is written to shared memory.  Executed by one whole warp.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
