@@ -215,7 +215,9 @@ struct cai_ctx {
   void* wt = nullptr;    // tile-major packed copy of W (pack_w_tiles_kernel), pair kernel
   CUtensorMap tm_a{};    // compact gathered rows in 128-row boxes (pair kernel)
   PairRowMaps tm_rows{};  // ... in 16-, 32-, ..., 128-row boxes (swapped pair kernel)
-  CUtensorMap tm_w{};    // wt as [2 n_vt (H / 64) 128, 64], 16 KiB unswizzled boxes
+  CUtensorMap tm_w{};    // wt as [pair_w_rows, 64], unswizzled boxes of 128 rows
+  CUtensorMap tm_w1{};   // ... and of pair_th1 rows (steps of one row tile)
+  int pair_th1 = 0;      // vocabulary rows per CTA and tile of those steps (pair_tile_rows)
   bool use_pair = false; // steps with >= pair_min_M rows run lm_head_pair_kernel
   int swap_max_n = 0;       // ... swapped when its tile width is at most this (pair_swapped)
   bool head_in_step = true; // the swapped-operand kernel is launched in multi-kernel steps
@@ -225,7 +227,7 @@ struct cai_ctx {
   float* inv_r = nullptr;  // [rows_cap] 1 / sqrt(mean h^2 + eps) of this step's rows
   __nv_bfloat16* h_prev = nullptr;  // [B P, H] previous step's rows (CAI_DIAGNOSTICS)
   void (*head_kernel)(CUtensorMap, HeadParams) = nullptr;
-  void (*pair_kernel)(CUtensorMap, CUtensorMap, PairRowMaps, PairParams) = nullptr;
+  void (*pair_kernel)(CUtensorMap, CUtensorMap, CUtensorMap, PairRowMaps, PairParams) = nullptr;
   int pair_min_M = 0, pair_grid = 0, pair_stages = 0, n_vt = 0, reduce_grid = 0;
   // Most pair stages in flight: swapped stages cut to size would give up to
   // 10 for narrow tiles, but beyond 8 the narrowest steps slow down again
@@ -475,8 +477,12 @@ int launch_pair_head(cai_ctx* c, int t, cudaStream_t stream) {
   pp.n_stages = c->pair_stages;
   pp.inv_r = c->inv_r;
   pp.ring_max = c->pair_ring_max;
+  pp.th1 = c->pair_th1;
+  pp.n_vt1 = (cfg.V + 2 * c->pair_th1 - 1) / (2 * c->pair_th1);
+  pp.w_dy = pair_w_run(cfg.V, c->pair_th1);
+  pp.w_ry = c->pair_th1 == kPairHalf ? cfg.H / kPairBlockK : 1;
   if (launch_pdl(c->pdl, c->pair_kernel, c->pair_grid, kPairThreads, c->pair_smem, stream,
-                 c->tm_a, c->tm_w, c->tm_rows, pp) != cudaSuccess)
+                 c->tm_a, c->tm_w, c->tm_w1, c->tm_rows, pp) != cudaSuccess)
     return check_launch(c);
   c->stats.launches++;
   if (c->need_reduce) {
@@ -919,6 +925,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     const int cset = env_int("CAI_PAIR_CLUSTERS");
     if (cset > 0 && cset < clusters) clusters = cset;
     c->pair_grid = 2 * clusters;
+    c->pair_th1 = pair_tile_rows(cfg->V, clusters);
     // Steps whose row-tile count does not divide the pairs leave one partial
     // per row and vocabulary tile to the reduce kernel; if no step size up to
     // B P does, that kernel is never launched.
@@ -973,7 +980,9 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   }
   CAI_ALLOC(c->part, float4, static_cast<size_t>(c->rows_cap) * part_cols)
   if (c->use_pair) {
-    CAI_ALLOC(c->wt, uint8_t, static_cast<size_t>(2 * c->n_vt) * kPairHalf * 2 * cfg->H)
+    CAI_ALLOC(c->wt, uint8_t,
+              static_cast<size_t>(pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1))) *
+                  kPairBlockK * 2)
     CAI_ALLOC(c->rowres, float4, c->rows_cap)
   }
   CAI_ALLOC(c->hidden_stage, uint8_t, static_cast<size_t>(c->BP) * cfg->H * 2)
@@ -1050,7 +1059,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     if (c->use_pair)
       pack_w_tiles_kernel<<<4 * sms, 256, 0, static_cast<cudaStream_t>(stream)>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wt), cfg->V, cfg->H,
-          static_cast<long long>(2 * c->n_vt) * kPairHalf * cfg->H / 8, g_dev);
+          pair_w_run(cfg->V, c->pair_th1),
+          pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1)) * (kPairBlockK / 8), g_dev);
     const cudaError_t e1 = cudaGetLastError();
     const cudaError_t e2 = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
     if (w_tmp) cudaFree(w_tmp);
@@ -1075,9 +1085,12 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
       (c->use_pair && !make_map(&c->tm_a, c->hc, c->rows_cap, cfg->H, kPairHalf)) ||
       (c->swap_max_n && !make_row_maps(c, cfg->H)) ||
       (c->use_pair &&
-       !make_map(&c->tm_w, c->wt, static_cast<uint64_t>(2 * c->n_vt) * (cfg->H / kPairBlockK) *
-                                      kPairHalf,
-                 kPairBlockK, kPairHalf, CU_TENSOR_MAP_SWIZZLE_NONE))) {
+       (!make_map(&c->tm_w, c->wt,
+                  pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1)), kPairBlockK,
+                  kPairHalf, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !make_map(&c->tm_w1, c->wt,
+                  pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1)), kPairBlockK,
+                  c->pair_th1, CU_TENSOR_MAP_SWIZZLE_NONE)))) {
     release(c);
     delete c;
     return CAI_ERR_CUDA;

@@ -13,8 +13,8 @@
 // tensor memory.  Per K block a CTA loads 32 KiB (16 KiB of hidden rows,
 // 16 KiB of W) for 2 * 128 * 256 * 64 flops, half the shared-memory traffic
 // per flop of a single-CTA 128 x 256 tile.  A tensor-memory lane holds one
-// row's logits, so the epilogue is a serial online softmax per thread over
-// the 256 columns of a tile, no shuffles.
+// row's logits, so the epilogue is a serial online softmax per thread, no
+// shuffles; two warps share a row's columns.
 //
 // Swapped, for narrow steps: the vocabulary fills the MMA M dimension (256
 // rows per pair, 128 per CTA: the W half is the A operand) and the masked
@@ -22,15 +22,22 @@
 // tiles of equal width N (a multiple of 32, at most 256), so a step pads at
 // most 31 rows per tile instead of up to 255: M = 305 runs as two 160-column
 // tiles, M = 159 as one of 160, M = 5 as one of 32.  A tensor-memory lane
-// then holds one vocabulary row of every column; the epilogue reduces across
-// lanes (transpose_logits32) and across the four epilogue warps (a
-// shared-memory exchange), and each CTA writes the triples of its 128
+// then holds one vocabulary row of every column; the epilogue reads fragments
+// in which a thread holds four vocabulary rows of a column, folds them into a
+// running triple per column over all of the pair's tiles, and merges across
+// lanes and warps once, at the end (every tile, when a pair's tiles have
+// different row tiles).  Each CTA writes the triples of its half of the
 // vocabulary rows: two partials per pair.  Each CTA loads N / 2 of a tile's
-// rows per K block as one box of exactly that many rows.  The cross-lane
-// reduction costs more than the serial one, so wide tiles stay unswapped: a
-// step runs swapped when N is at most swap_max_n (192 by default; measured
-// per step on the Dream shape: N = 64..192 3 to 11 % faster than the padded
-// unswapped tile, N = 224, 256 1 to 7 % slower).
+// rows per K block as one box of exactly that many rows.  A step runs swapped
+// when N is at most swap_max_n (192 by default).
+//
+// The epilogue of a pair's last tile is not hidden by anything.  With one warp
+// per quarter and a 31-merge transposition per tile it took 6 us at N = 96 and
+// 12 us at N = 192 after the last copy, and it bounded whole steps of models
+// with a short K (22000 x 1024, M = 192: 37.4 us a step, now 25.7; M = 352
+// 48.1 -> 27.9; unswapped M = 224 27.9 -> 21.9).  At 4096 x 126464 a step takes
+// 165.8 us instead of 172.5 at M = 192, 245 instead of 254.6 at M = 352 (these
+// with the set-up below).
 //
 // Partials: when the number of pairs is a multiple of the number of row
 // tiles n_rt, every tile of a pair has the same row tile, and the epilogue
@@ -45,13 +52,15 @@
 // and by the n_rt pairs of its row tiles from L2; the gathered hidden rows
 // (at most 2 x 65536 x 16384 bytes, in practice tens of MB) stay in L2.
 //
-// Roles per CTA (192 threads): warp 0 producer (hidden half and W half by
-// TMA; W from a tile-major packed copy in which every box is one contiguous
-// 16 KiB block); warp 1 allocates tensor memory and, in the even CTA, issues
-// the MMAs; warps 2..5 epilogue.  Both CTAs' copies of a stage complete on
+// Roles per CTA (320 threads): warp 0 producer (hidden half and W half by
+// TMA; W from a packed copy in which every box is one contiguous block, or
+// kStatic from the caller's rows); warp 1 allocates tensor memory and, in the
+// even CTA, issues the MMAs; warps 2..9 epilogue.  Both CTAs' copies of a stage complete on
 // the even CTA's barrier (cta_group::2 loads), which the even CTA's producer
 // arms with the bytes of both.  Two accumulator buffers let the epilogue of
-// one tile overlap the next tile's MMAs.
+// one tile overlap the next tile's MMAs.  Barriers, tensor memory and map
+// prefetches come before the dependency wait, so that a step's first copies
+// start right after the gather.
 //
 // How stages are issued.  The producer and the MMA warp run their loops with
 // all 32 lanes, every loop bound and descriptor the same in each, and only the
@@ -82,7 +91,10 @@
 
 namespace cai {
 
-constexpr int kPairThreads = 192;
+constexpr int kPairEpiWarps = 8;      // two per tensor-memory quarter, half of the columns each
+constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;
+// Registers a thread: a gather CTA (256 threads of at most 56) fits beside a pair CTA.
+constexpr int kPairRegs = 160;
 constexpr int kPairTileRows = 256;    // masked rows per pair tile (MMA M)
 constexpr int kPairTileVocab = 256;   // vocabulary rows per pair tile (MMA N)
 constexpr int kPairHalf = 128;        // rows of each per CTA
@@ -92,6 +104,7 @@ constexpr int kPairStageBytes = 2 * kPairHalfBytes;          // A half + B half
 constexpr int kPairTmemCols = 2 * kPairTileVocab;            // two accumulators
 constexpr int kSwapColStep = 32;    // swapped orientation: granularity of N
 constexpr int kSwapXchBytes = 2 * 4 * kPairTileVocab * 16;  // cross-warp exchange, two buffers
+constexpr int kSwapChunks = kPairTileVocab / 32;  // most 16-column chunks of an epilogue warp
 constexpr int kPairMaxRing = 12;    // swapped stages are cut to size: up to this many
 
 // Tensor maps of the gathered rows with boxes of 16, 32, ..., 128 rows
@@ -115,6 +128,10 @@ struct PairParams {
   int n_stages;
   const float* inv_r;  // final-norm row scales [rows] (kNorm only)
   int ring_max;        // most stages in flight (<= kPairMaxRing)
+  int M_fixed;         // kStatic: rows of this launch
+  int th1, n_vt1;      // steps of one row tile: vocabulary rows per CTA and tile, tiles
+  // W map coordinates of K block kb, vocabulary row r (a tile's first): (kb w_dx, r w_ry + kb w_dy).
+  int w_dx, w_dy, w_ry;
 };
 
 // Row tiles of a pair step with M rows (both orientations).
@@ -145,30 +162,56 @@ __host__ __device__ inline int pair_partials_per_row(int M, int n_pairs, bool sw
   return (swap ? 2 : 1) * (n_pairs / n_rt);
 }
 
-__host__ __device__ inline size_t pair_smem_bytes(int n_stages, bool swap) {
-  return 1024 + static_cast<size_t>(n_stages) * kPairStageBytes + (swap ? kSwapXchBytes : 0) +
-         static_cast<size_t>(2 * kPairMaxRing + 7) * 8 + 16;
+// Vocabulary rows per CTA and tile of a step of one row tile: such a step is
+// bound by reading W, so V is dealt out evenly, every pair the same number n
+// of tiles of equal height (a multiple of 8 rows, the swizzle atom, at most
+// 128).
+__host__ __device__ inline int pair_even_rows(int V, int n_pairs) {
+  const int n = (V + 2 * kPairHalf * n_pairs - 1) / (2 * kPairHalf * n_pairs);
+  const int per = (V + 2 * n_pairs * n - 1) / (2 * n_pairs * n);
+  return (per + 7) / 8 * 8;
 }
 
-// Pack W [V, H] (row-major bf16) tile-major for the pair kernel: 128-row
-// tile t, K block kb is the 16 KiB block at (t * (H / 64) + kb) * 16 KiB, in
-// the 128-byte-swizzled K-major layout (row r's 16-byte chunk c at
-// r * 128 + (c ^ (r & 7)) * 16).  Rows >= V are zero; n_tiles = 2 n_vt.  The
-// kernel reads it through a tensor map of [2 n_vt (H / 64) 128, 64] bf16 with
-// 64 x 128 boxes and no swizzle: box (t (H / 64) + kb) is that block.
+// ... of a context, whose packed W then has the matching order (pair_w_run).
+// From five tiles a pair on, 128-row tiles are kept: pairs that finish early
+// leave their share of the memory bandwidth to the others, and the order that
+// even tiles need reads 128-row tiles a little slower.  Measured, microseconds
+// a step: 22000 x 1024 (n = 2), M = 224 28.3 -> 25.5 with even tiles; 126464 x
+// 4096 (n = 7), M = 128 165.7 -> 163.8, but M = 264 232.7 -> 236.
+__host__ __device__ inline int pair_tile_rows(int V, int n_pairs) {
+  return V > 4 * 2 * kPairHalf * n_pairs ? kPairHalf : pair_even_rows(V, n_pairs);
+}
+
+__host__ __device__ inline size_t pair_smem_bytes(int n_stages, bool swap) {
+  return 1024 + static_cast<size_t>(n_stages) * kPairStageBytes + (swap ? kSwapXchBytes : 0) +
+         static_cast<size_t>(2 * kPairMaxRing + 9) * 8 + 16 + 3 * kPairHalf * 4;
+}
+
+// Pack W [V, H] (row-major bf16) for the pair kernel in blocks of `run` rows x
+// 64 columns, the K blocks of a run one after the other; each row's 128 bytes
+// with the 128-byte swizzle of 8-row atoms (16-byte chunk c of row r at
+// c ^ (r & 7)); rows >= V zero.  The kernel reads it through a tensor map of
+// 64 columns with no swizzle: K block kb of row r (r / run = q) is map row
+// q run KB + kb run + r - q run.  Two runs are used (pair_w_run):
+//   128, when every tile is 128 rows high: a tile's K blocks are contiguous;
+//   all round8(V) rows, otherwise: any run of 8-row atoms of a K block is one
+//   contiguous block, so steps of one row tile may cut V evenly (pair_even_rows)
+//   and wider ones in 128-row tiles.  Reading 128-row tiles in this order is
+//   0.6 % slower (152064 x 3584, M = 96: 169.2 us a step against 170.5).
 __global__ void pack_w_tiles_kernel(const uint4* __restrict__ W, uint4* __restrict__ out, int V,
-                                    int H, long long n_chunks, const __nv_bfloat16* __restrict__ gw) {
+                                    int H, int run, long long n_chunks,
+                                    const __nv_bfloat16* __restrict__ gw) {
   const int KB = H / kPairBlockK;
-  const long long tile_chunks = static_cast<long long>(KB) * (kPairHalfBytes / 16);
+  const long long run_rows = static_cast<long long>(run) * KB;
   for (long long d = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; d < n_chunks;
        d += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long t = d / tile_chunks;
-    const int rem = static_cast<int>(d - t * tile_chunks);
-    const int kb = rem / (kPairHalfBytes / 16);
-    const int inblk = rem % (kPairHalfBytes / 16);  // 16-byte chunk in the block
-    const int r = inblk >> 3;
-    const int cl = (inblk & 7) ^ (r & 7);
-    const long long v = t * kPairHalf + r;
+    const long long row = d >> 3;
+    const long long q = row / run_rows;
+    const long long rem = row - q * run_rows;
+    const int kb = static_cast<int>(rem / run);
+    const int r = static_cast<int>(rem - static_cast<long long>(kb) * run);
+    const long long v = q * run + r;
+    const int cl = static_cast<int>(d & 7) ^ (r & 7);
     uint4 val = make_uint4(0u, 0u, 0u, 0u);
     if (v < V) val = W[(v * H + static_cast<long long>(kb) * kPairBlockK) / 8 + cl];
     if (gw) val = scale_chunk(val, gw + kb * kPairBlockK + cl * 8);
@@ -176,15 +219,25 @@ __global__ void pack_w_tiles_kernel(const uint4* __restrict__ W, uint4* __restri
   }
 }
 
+// Rows per run of the packed W, and its rows of 64 columns.
+__host__ __device__ inline int pair_w_run(int V, int th1) {
+  return th1 == kPairHalf ? kPairHalf : (V + 7) / 8 * 8;
+}
+__host__ __device__ inline long long pair_w_rows(int V, int H, int run) {
+  return static_cast<long long>((V + run - 1) / run) * run * (H / kPairBlockK);
+}
+
 struct PairSmem {
   uint8_t* stage;      // n_stages x kPairStageBytes: the ring (A half, B half per stage)
-  float4* xch;         // swapped orientation: 2 x [4 warps][256 columns] triples
+  float4* xch;         // swapped orientation: 2 x [4 quarters][256 columns] triples
   uint64_t* full;      // kPairMaxRing (even CTA): both CTAs' halves of the stage landed
   uint64_t* empty;     // kPairMaxRing: the pair's MMAs are done with the stage
   uint64_t* accf;      // 2: accumulator ready
   uint64_t* acce;      // 2 (even CTA): accumulator drained by both epilogues
   uint64_t* drain;     // 1 (even CTA): abort path, issued MMAs complete
-  uint64_t* xchb;      // 2 (swapped): the four epilogue warps wrote xch[buffer]
+  uint64_t* xchb;      // 2 (swapped): the epilogue warps wrote xch[buffer]
+  uint64_t* xcub;      // 2 (unswapped): the odd half's warps wrote xchu, the even half's read it
+  float* xchu;         // unswapped orientation: [3][128] triples of the odd half
   uint32_t* tmem_slot;
   volatile int* abort;
 };
@@ -203,8 +256,10 @@ __device__ __forceinline__ PairSmem pair_carve(uint8_t* raw, int n_stages, bool 
   s.acce = s.accf + 2;
   s.drain = s.acce + 2;
   s.xchb = s.drain + 1;
-  s.tmem_slot = reinterpret_cast<uint32_t*>(s.xchb + 2);
+  s.xcub = s.xchb + 2;
+  s.tmem_slot = reinterpret_cast<uint32_t*>(s.xcub + 2);
   s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
+  s.xchu = reinterpret_cast<float*>(s.tmem_slot + 4);
   return s;
 }
 
@@ -232,10 +287,14 @@ __device__ __forceinline__ void pair_drain(uint64_t* bar, uint32_t parity, uint3
 // kNorm: as in lm_head_softmax_kernel, row n's logits are scaled by inv_r[n]
 // (written by the gather).  Swapped steps (pair_swapped) load a tile's rows
 // through hm instead of tm_a.
-template <bool kNorm>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+// kStatic: M_fixed rows that the caller passes, known at launch (M <= 256, W
+// row-major through the map's own swizzle); the set-up then comes before the
+// dependency wait.
+template <bool kNorm, bool kStatic = false>
+__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
     lm_head_pair_kernel(const __grid_constant__ CUtensorMap tm_a,
                         const __grid_constant__ CUtensorMap tm_w,
+                        const __grid_constant__ CUtensorMap tm_w1,
                         const __grid_constant__ PairRowMaps hm, const PairParams p) {
   extern __shared__ uint8_t smem_raw[];
   const int warp = threadIdx.x >> 5;
@@ -244,23 +303,62 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const int pair = blockIdx.x >> 1;
   const int n_pairs = gridDim.x >> 1;
 
-  grid_dependency_wait();    // d_M and the gathered rows of this step
+  // Set-up that does not depend on M, before the dependency wait.
+  PairSmem sm = pair_carve(smem_raw, p.n_stages, p.swap_max_n > 0);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kPairMaxRing; ++s) {
+      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&sm.accf[a], 1);
+      mbar_init(&sm.acce[a], 2 * kPairEpiWarps);  // the epilogue warps of both CTAs
+      mbar_init(&sm.xchb[a], kPairEpiWarps);      // the epilogue warps of this CTA
+      mbar_init(&sm.xcub[a], kPairEpiWarps / 2);  // ... of one half of the columns
+    }
+    mbar_init(sm.drain, 1);
+    *sm.abort = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tm_a);
+    prefetch_tmap(&tm_w);
+    prefetch_tmap(&tm_w1);
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(sm.tmem_slot, kPairTmemCols);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  cluster_sync();  // barriers of both CTAs initialised, tensor memory allocated
+  tc_fence_after();
+  const uint32_t tmem_base = *sm.tmem_slot;
+
+  int M;
+  if constexpr (kStatic) {
+    M = p.M_fixed;
+    grid_dependency_wait();  // the caller's rows and W, the scratch
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.err[1] = 0u;  // the merge's ticket
+  } else {
+    grid_dependency_wait();  // d_M and the gathered rows of this step
+    M = *p.d_M;
+  }
   // Every thread (the CTA counts once all of them have), after the wait: the
   // commit kernel, which may start from here, reads the previous step's state
   // before waiting for this kernel.
   grid_launch_dependents();
-  const int M = *p.d_M;
   if (p.m_hist_slot && blockIdx.x == 0 && threadIdx.x == 0 && (M >= p.min_M || p.min_M <= 1))
     *p.m_hist_slot = M;
-  if (M < p.min_M || M < 1) return;  // both CTAs of every pair take the same branch
+  // Nothing to decode here: no tiles, every role falls through.
+  const bool none = M < p.min_M || M < 1;
   const bool swap = pair_swapped(M, p.swap_max_n);  // the same in every CTA
 
-  PairSmem sm = pair_carve(smem_raw, p.n_stages, p.swap_max_n > 0);
   const int KB = p.H / kPairBlockK;
-  const int n_rt = pair_row_tiles(M);
+  const int n_rt = none ? 1 : pair_row_tiles(M);
   // Rows per row tile: 256 (the MMA M of the pair), or N when swapped.
   const int rt_rows = swap ? swap_tile_cols(M, n_rt) : kPairTileRows;
-  const int n_tiles = p.n_vt * n_rt;
+  // Vocabulary rows per CTA and tile (half: MMA columns per CTA when unswapped).
+  const int th = n_rt == 1 ? p.th1 : kPairHalf;
+  const int half = (th + 31) & ~31;
+  const int n_tiles = none ? 0 : n_rt == 1 ? p.n_vt1 : p.n_vt * n_rt;
   const int my_tiles = pair < n_tiles ? (n_tiles - pair + n_pairs - 1) / n_pairs : 0;
   // Swapped stages hold the W half and one box of rows_tile / 2 rows, so the
   // ring (n_stages slots of kPairStageBytes) is re-cut to that size: more
@@ -271,40 +369,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const int ring_bytes =
       p.n_stages * kPairStageBytes + (!swap && p.swap_max_n > 0 ? kSwapXchBytes : 0);
   const int n_ring = min(p.ring_max, ring_bytes / stage_stride);
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < n_ring; ++s) {
-      mbar_init(&sm.full[s], 1);
-      mbar_init(&sm.empty[s], 1);
-    }
-    for (int a = 0; a < 2; ++a) {
-      mbar_init(&sm.accf[a], 1);
-      mbar_init(&sm.acce[a], 8);  // four epilogue warps in each CTA
-    }
-    mbar_init(sm.drain, 1);
-    if (swap) {
-      mbar_init(&sm.xchb[0], 4);  // the four epilogue warps of this CTA
-      mbar_init(&sm.xchb[1], 4);
-    }
-    *sm.abort = 0;
-    fence_mbar_init();
-  }
-  if (warp == 0 && lane == 0) {
-    prefetch_tmap(&tm_w);
-    if (swap) {
-      prefetch_tmap(&hm.box[swap_tile_cols(M, n_rt) / 32 - 1]);
-    } else {
-      prefetch_tmap(&tm_a);
-    }
-  }
-  if (warp == 1) {
-    tmem_alloc_pair(sm.tmem_slot, kPairTmemCols);
-    tmem_relinquish_pair();
-  }
-  tc_fence_before();
-  cluster_sync();  // barriers of both CTAs initialised, tensor memory allocated
-  tc_fence_after();
-  const uint32_t tmem_base = *sm.tmem_slot;
 
   if (warp == 0) {
     // -------------------------------------------------------- producer --
@@ -319,14 +383,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     const int box_rows = rt_rows / 2;
     // Bytes of one stage, both CTAs (the even CTA arms its barrier for them).
     const uint32_t stage_tx =
-        swap ? 2u * static_cast<uint32_t>(kPairHalfBytes + box_rows * kPairBlockK * 2)
-              : 2u * kPairStageBytes;
+        2u * static_cast<uint32_t>((th + (swap ? box_rows : kPairHalf)) * kPairBlockK * 2);
+    const CUtensorMap* tmw = n_rt == 1 ? &tm_w1 : &tm_w;
     for (int i = 0; i < my_tiles && ok; ++i) {
       const int t = pair + i * n_pairs;
       const int v = t / n_rt, j = t - v * n_rt;
       // First row of this CTA's half of the tile's rows.
       const int a_row = j * rt_rows + static_cast<int>(rank) * (swap ? rt_rows / 2 : kPairHalf);
-      const int w_box = (2 * v + static_cast<int>(rank)) * KB;
+      const int w_row = (2 * v + static_cast<int>(rank)) * th;
       for (int kb = 0; kb < KB; ++kb) {
         ok = ok && mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
         if (leader && ok) {
@@ -337,11 +401,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           if (rank == 0) mbar_arrive_expect_tx(&sm.full[r.slot], stage_tx);
           if (swap) {
             // A: the W half; B: the CTA's rows, one box of box_rows.
-            tma_load_2d_pair_nohint(dst, &tm_w, bar, 0, (w_box + kb) * kPairHalf);
+            tma_load_2d_pair_nohint(dst, tmw, bar, kb * p.w_dx, w_row * p.w_ry + kb * p.w_dy);
             tma_load_2d_pair(dst + kPairHalfBytes, &hm.box[q1], bar, kb * kPairBlockK, a_row, pol_a);
           } else {
             tma_load_2d_pair(dst, &tm_a, bar, kb * kPairBlockK, a_row, pol_a);
-            tma_load_2d_pair_nohint(dst + kPairHalfBytes, &tm_w, bar, 0, (w_box + kb) * kPairHalf);
+            tma_load_2d_pair_nohint(dst + kPairHalfBytes, tmw, bar, kb * p.w_dx,
+                                    w_row * p.w_ry + kb * p.w_dy);
           }
         }
         __syncwarp();
@@ -360,9 +425,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     if (rank == 0) {
       // -------------------------------------------- MMA issuer (even CTA) --
       // Swapped: M = 256 vocabulary rows, N = the tile's rows; else M = 256
-      // rows, N = 256 vocabulary rows.
-      const uint32_t idesc =
-          idesc_bf16_f32(256, swap ? static_cast<uint32_t>(rt_rows) : kPairTileVocab);
+      // rows, N = 2 half vocabulary rows.
+      const uint32_t idesc = idesc_bf16_f32(256, static_cast<uint32_t>(swap ? rt_rows : 2 * half));
       const bool leader = elect_one();
       const uint64_t desc0 = sdesc_k_sw128(smem_addr(sm.stage));
       PairRing r;
@@ -402,55 +466,74 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     __syncwarp();
   } else if (swap) {
     // ----------------------------------------------- epilogue (swapped) --
-    // Lane l of warp `quarter` holds vocabulary row 256 v + 128 rank + 32
-    // quarter + l of all rt_rows columns (the tile's rows).  Per 32 columns the
-    // warp's 32 rows are merged across lanes (lane l then holds column l), the
-    // four warps' slices through xch, and thread et of the four warps keeps
-    // columns et and et + 128.
+    // The CTA's 128 accumulator lanes are vocabulary rows, its rt_rows columns
+    // the tile's rows.  A warp holds 32 lanes and half of the columns, 16 at a
+    // time: with 16x256b loads thread (g = lane / 4, h = lane % 4) gets the
+    // four lanes g, g + 8, g + 16, g + 24 of the columns 8 j + 2 h + e, and
+    // folds them into a running triple per column over all of the pair's
+    // tiles.  Only at the end are the eight threads of a column merged
+    // (transposing butterfly) and the four warps of a column (through xch).
     const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. 32 quarter + 31
-    const int ew = warp - 2;       // 0..3: slot in the cross-warp exchange
-    const int et = ew * 32 + lane;
+    const int et = threadIdx.x - 64;
+    const int col_half = ((warp - 2) >> 2) * (rt_rows / 2);
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t acce_remote = mapa_shared(sm.acce, 0);
     const int per_row = pair_partials_per_row(M, n_pairs, true);  // > 0: two partials per pair
-    const int nch = rt_rows / 32;
-    float am[2] = {kNegBig, kNegBig}, as[2] = {0.0f, 0.0f};
-    int aix[2] = {INT_MAX, INT_MAX};
+    const int nch = rt_rows / 32;  // 16-column chunks of this warp
+    const int g = lane >> 2, h2 = 2 * (lane & 3);
+    float am[4 * kSwapChunks], as[4 * kSwapChunks];
+    int aix[4 * kSwapChunks];
     for (int i = 0; i < my_tiles; ++i) {
       const int t = pair + i * n_pairs;
       const int v = t / n_rt, j = t - v * n_rt;
+      const int row0 = j * rt_rows;
       const int acc = i & 1;
+      // This thread's vocabulary rows; those past the tile (stale stage bytes)
+      // or past V count as -inf.
+      const int vbase = (2 * v + static_cast<int>(rank)) * th;
+      const int vrow = vbase + quarter * 32 + g;
+      const int nrow = min(vbase + th, p.V) - vrow;  // rows 8 k < nrow exist
+      const bool whole = nrow > 24;
+      if (i == 0 || per_row == 0) {
+#pragma unroll
+        for (int k = 0; k < 4 * kSwapChunks; ++k) {
+          am[k] = kNegBig;
+          as[k] = 0.0f;
+          aix[k] = nrow > 0 ? vrow : INT_MAX;
+        }
+      }
       if (!mbar_wait(&sm.accf[acc], (i >> 1) & 1, sm.abort, p.err, kErrWaitAccFull)) break;
       tc_fence_after();
-      const uint32_t tbase = tmem_base + lane_base + static_cast<uint32_t>(acc * kPairTileVocab);
-      const int vrow = v * kPairTileVocab + static_cast<int>(rank) * kPairHalf + quarter * 32 + lane;
-      const bool valid = vrow < p.V;  // vocabulary rows past V are zero padding
-      const bool pvalid = (vrow ^ 16) < p.V;
-      const int row0 = j * rt_rows;
-      // Buffer i & 1 is written again at tile i + 2, after every warp has
-      // arrived for tile i + 1, which each does after reading tile i.  One
-      // chunk of 32 columns at a time (the reduction is not unrolled over
-      // chunks: its code stays small enough for the instruction cache).
-      float4* xb = sm.xch + (i & 1) * 4 * kPairTileVocab;
-#pragma unroll 1
-      for (int c = 0; c < nch; ++c) {
-        uint32_t x[32];
-        tmem_ld_32cols(tbase + static_cast<uint32_t>(32 * c), x);
-        tmem_ld_wait();
-        float z[32];
+      const uint32_t tbase = tmem_base + lane_base +
+                             static_cast<uint32_t>(acc * kPairTileVocab + col_half);
+      uint32_t xa[16], xb[16];
+      tmem_ld_16cols_frag(tbase, xa);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          float sc = kLog2e;
-          if constexpr (kNorm) {
-            const int row = row0 + 32 * c + k;
-            if (row < M) sc = kLog2e * __ldg(p.inv_r + row);
+      for (int c = 0; c < kSwapChunks; ++c) {
+        if (c < nch) {
+          uint32_t(&x)[16] = (c & 1) ? xb : xa;
+          tmem_ld_wait16(x);
+          if (c + 1 < kSwapChunks && c + 1 < nch)
+            tmem_ld_16cols_frag(tbase + static_cast<uint32_t>(16 * (c + 1)), (c & 1) ? xa : xb);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {  // column 8 (q / 2) + h2 + q % 2 of the chunk
+            float sc = kLog2e;
+            if constexpr (kNorm) {
+              const int row = row0 + col_half + 16 * c + 8 * (q >> 1) + h2 + (q & 1);
+              if (row < M) sc = kLog2e * __ldg(p.inv_r + row);
+            }
+            float z[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              z[k] = __fmul_rn(__uint_as_float(x[8 * (k >> 1) + 4 * (q >> 1) + 2 * (k & 1) + (q & 1)]),
+                               sc);
+            if (!whole) {
+#pragma unroll
+              for (int k = 0; k < 4; ++k) z[k] = 8 * k < nrow ? z[k] : -INFINITY;
+            }
+            fold4(am[4 * c + q], as[4 * c + q], aix[4 * c + q], z, vrow);
           }
-          z[k] = valid ? __uint_as_float(x[k]) * sc : kNegBig;
         }
-        float m, s;
-        int ix;
-        transpose_logits32(z, valid, pvalid, vrow, lane, m, s, ix);
-        xb[ew * kPairTileVocab + 32 * c + lane] = make_float4(m, s, __int_as_float(ix), 0.0f);
       }
       tc_fence_before();
       __syncwarp();
@@ -460,92 +543,92 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         else
           mbar_arrive_cluster(acce_remote + static_cast<uint32_t>(acc * 8));
       }
-      if (lane == 0) mbar_arrive(&sm.xchb[i & 1]);
-      if (!mbar_wait(&sm.xchb[i & 1], (i >> 1) & 1, sm.abort, p.err, kErrWaitEpi)) break;
+      if (per_row > 0 && i + 1 < my_tiles) continue;
+      // One partial per column, of this tile (buffer i & 1 is written again at
+      // tile i + 2, after every warp has arrived for tile i + 1, which each
+      // does after reading tile i) or, with per_row > 0, of all tiles.
+      const int buf = per_row > 0 ? 0 : i & 1;
+      float4* xch = sm.xch + buf * 4 * kPairTileVocab + quarter * kPairTileVocab + col_half;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int col = et + 128 * h;
-        if (col < rt_rows) {
-          float m = kNegBig, s = 0.0f;
-          int ix = INT_MAX;
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const float4 a = xb[w * kPairTileVocab + col];
-            merge_tri(m, s, ix, a.x, a.y, __float_as_int(a.z));
-          }
-          const int row = row0 + col;
-          if (per_row > 0)
-            merge_tri(am[h], as[h], aix[h], m, s, ix);
-          else if (row < M && CAI_IN_RANGE(v < p.n_vt, p.err))
-            p.part[static_cast<size_t>(row) * (2 * p.n_vt) + 2 * v + static_cast<int>(rank)] =
-                make_float4(m, s, __int_as_float(ix), 0.0f);
+      for (int c = 0; c < kSwapChunks; ++c) {
+        if (c < nch) {
+          float4 f;
+          merge_frag8(am + 4 * c, as + 4 * c, aix + 4 * c, lane, f);
+          if ((lane & 4) == 0)
+            xch[16 * c + ((lane & 16) ? 8 : 0) + h2 + ((lane & 8) ? 1 : 0)] = f;
         }
       }
-    }
-    if (per_row > 0) {
-      // The pair's row tile is fixed (pair mod n_rt); a pair without tiles
-      // writes the empty triple.
-      const int row0 = (pair % n_rt) * rt_rows;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.xchb[buf]);
+      if (!mbar_wait(&sm.xchb[buf], per_row > 0 ? 0u : (i >> 1) & 1, sm.abort, p.err, kErrWaitEpi))
+        break;
+      if (et < rt_rows && row0 + et < M) {
+        float m = kNegBig, sum = 0.0f;
+        int ix = INT_MAX;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int col = et + 128 * h;
-        if (col < rt_rows && row0 + col < M)
-          p.part[static_cast<size_t>(row0 + col) * per_row + 2 * (pair / n_rt) +
-                 static_cast<int>(rank)] = make_float4(am[h], as[h], __int_as_float(aix[h]), 0.0f);
+        for (int w = 0; w < 4; ++w) {
+          const float4 a = sm.xch[(buf * 4 + w) * kPairTileVocab + et];
+          merge_tri(m, sum, ix, a.x, a.y, __float_as_int(a.z));
+        }
+        // Valid rows but no logit above the empty maximum (all -inf): no softmax.
+        if (m == kNegBig && ix != INT_MAX) sum = __int_as_float(0x7fc00000);
+        const size_t row = static_cast<size_t>(row0 + et);
+        if (per_row > 0)
+          p.part[row * per_row + 2 * (pair / n_rt) + static_cast<int>(rank)] =
+              make_float4(m, sum, __int_as_float(ix), 0.0f);
+        else if (CAI_IN_RANGE(v < p.n_vt, p.err))
+          p.part[row * (2 * p.n_vt) + 2 * v + static_cast<int>(rank)] =
+              make_float4(m, sum, __int_as_float(ix), 0.0f);
       }
+    }
+    if (per_row > 0 && my_tiles == 0 && !none) {
+      // A pair without tiles writes the empty triple for its row tile.
+      const int row = (pair % n_rt) * rt_rows + et;
+      if (et < rt_rows && row < M)
+        p.part[static_cast<size_t>(row) * per_row + 2 * (pair / n_rt) + static_cast<int>(rank)] =
+            make_float4(kNegBig, 0.0f, __int_as_float(INT_MAX), 0.0f);
     }
   } else {
     // --------------------------------------------------------- epilogue --
+    // A tensor-memory lane holds one row's logits; the two warps of a quarter
+    // take half of the columns each (the even and the odd CTA's vocabulary
+    // rows) and merge their triples through xch.
     const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. 32 quarter + 31
+    const int odd = (warp - 2) >> 2;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t acce_remote = mapa_shared(sm.acce, 0);
     const int per_row = pair_partials_per_row(M, n_pairs, false);  // > 0: one partial per pair
-    float am = kNegBig, as = 0.0f;
-    int aix = INT_MAX;
+    float* xm = sm.xchu + quarter * 32 + lane;  // [3][128]: max, sum, index
+    float m = kNegBig, s = 0.0f;
+    int ix = INT_MAX;
     for (int i = 0; i < my_tiles; ++i) {
       const int t = pair + i * n_pairs;
       const int v = t / n_rt, j = t - v * n_rt;
       const int acc = i & 1;
+      if (per_row == 0) {
+        m = kNegBig;
+        s = 0.0f;
+        ix = INT_MAX;
+      }
       if (!mbar_wait(&sm.accf[acc], (i >> 1) & 1, sm.abort, p.err, kErrWaitAccFull)) break;
       tc_fence_after();
-      const uint32_t tbase = tmem_base + lane_base + static_cast<uint32_t>(acc * kPairTileVocab);
+      const uint32_t tbase = tmem_base + lane_base +
+                             static_cast<uint32_t>(acc * kPairTileVocab + odd * half);
       const int row = j * kPairTileRows + static_cast<int>(rank) * kPairHalf + quarter * 32 + lane;
       float rs = kLog2e;
       if constexpr (kNorm) {
         if (row < M) rs = kLog2e * __ldg(p.inv_r + row);
       }
-      const int vbase = v * kPairTileVocab;
-      float m = kNegBig, s = 0.0f;
-      int ix = INT_MAX;
+      // Columns [0, half) are the even CTA's th vocabulary rows, [half, 2 half)
+      // the odd one's; columns past th (stale stage bytes) or past V are left out.
+      const int vbase = (2 * v + odd) * th;
+      const int nrow = min(th, p.V - vbase);
 #pragma unroll 1
-      for (int c = 0; c < kPairTileVocab / 32; ++c) {
+      for (int c = 0; c < half / 32; ++c) {
         uint32_t x[32];
         tmem_ld_32cols(tbase + static_cast<uint32_t>(32 * c), x);
         tmem_ld_wait();
-        const int v0 = vbase + 32 * c;
-        const int nvalid = min(32, p.V - v0);  // vocabulary rows past V are zero padding
-        float cm = kNegBig;
-        int ci = 0;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const float z = __uint_as_float(x[k]) * rs;
-          if (k < nvalid && z > cm) {
-            cm = z;
-            ci = k;
-          }
-        }
-        if (cm > m) {  // strictly: an equal maximum keeps the lower index
-          s *= fast_exp2(m - cm);
-          m = cm;
-          ix = v0 + ci;
-        }
-        float cs = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const float z = __uint_as_float(x[k]) * rs;
-          cs += k < nvalid ? fast_exp2(z - m) : 0.0f;
-        }
-        s += cs;
+        fold_row32(m, s, ix, x, rs, vbase + 32 * c, nrow - 32 * c);
       }
       tc_fence_before();
       __syncwarp();
@@ -555,19 +638,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         else
           mbar_arrive_cluster(acce_remote + static_cast<uint32_t>(acc * 8));
       }
-      if (per_row > 0)
-        merge_tri(am, as, aix, m, s, ix);  // tiles in increasing v: ties keep the lower index
-      else if (row < M && CAI_IN_RANGE(v < p.n_vt, p.err))
-        p.part[static_cast<size_t>(row) * p.n_vt + v] = make_float4(m, s, __int_as_float(ix), 0.0f);
+      if (per_row > 0 && i + 1 < my_tiles) continue;
+      // n-th exchange of this step: the odd half's warps write it once the
+      // even half's have read the one before (xcub[1]), and announce it (xcub[0]).
+      const int n = per_row > 0 ? 0 : i;
+      if (odd) {
+        if (n > 0 && !mbar_wait(&sm.xcub[1], (n - 1) & 1, sm.abort, p.err, kErrWaitEpi)) break;
+        xm[0] = m;
+        xm[kPairHalf] = s;
+        xm[2 * kPairHalf] = __int_as_float(ix);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.xcub[0]);
+        continue;
+      }
+      if (!mbar_wait(&sm.xcub[0], n & 1, sm.abort, p.err, kErrWaitEpi)) break;
+      const float om = xm[0], os = xm[kPairHalf];
+      const int oix = __float_as_int(xm[2 * kPairHalf]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.xcub[1]);
+      merge_tri(m, s, ix, om, os, oix);
+      if (row < M) {
+        if (per_row > 0)
+          p.part[static_cast<size_t>(row) * per_row + pair / n_rt] =
+              make_float4(m, s, __int_as_float(ix), 0.0f);
+        else if (CAI_IN_RANGE(v < p.n_vt, p.err))
+          p.part[static_cast<size_t>(row) * p.n_vt + v] =
+              make_float4(m, s, __int_as_float(ix), 0.0f);
+      }
     }
-    if (per_row > 0) {
-      // The pair's row tile is fixed (pair mod n_rt); a pair without tiles
-      // writes the empty triple.
+    if (per_row > 0 && my_tiles == 0 && !none && !odd) {
+      // A pair without tiles writes the empty triple for its row tile.
       const int row = (pair % n_rt) * kPairTileRows + static_cast<int>(rank) * kPairHalf +
                       quarter * 32 + lane;
       if (row < M)
         p.part[static_cast<size_t>(row) * per_row + pair / n_rt] =
-            make_float4(am, as, __int_as_float(aix), 0.0f);
+            make_float4(kNegBig, 0.0f, __int_as_float(INT_MAX), 0.0f);
     }
   }
 

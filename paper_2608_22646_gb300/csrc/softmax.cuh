@@ -103,57 +103,83 @@ __device__ __forceinline__ void transpose_merge32(float (&m)[32], float (&s)[32]
   }
 }
 
-// 32 rows (one per lane) x 32 columns of logits z (log2 units) -> lane l
-// holds the (max, sum, argmax) of column l over the 32 rows, as
-// transpose_merge32 but with the first halving step specialised: a lane's
-// partner at width 16 holds vocabulary row vrow ^ 16, so only the logits are
-// exchanged (16 shuffles instead of 48).  vrow is this lane's vocabulary row
-// (lane-aligned: vrow % 32 == lane), valid / pvalid whether this lane's and
-// the partner's rows exist.  On return m[0], s[0], ix[0] hold the column's
-// triple; z is clobbered.
-__device__ __forceinline__ void transpose_logits32(float (&z)[32], bool valid, bool pvalid,
-                                                   int vrow, int lane, float& om, float& os,
-                                                   int& oi) {
-  float m[16], s[16];
-  int ix[16];
-  const bool up = (lane & 16) != 0;
-  const float ks = valid ? 1.0f : 0.0f, rs = pvalid ? 1.0f : 0.0f;
-  const int ki = valid ? vrow : INT_MAX, ri = pvalid ? (vrow ^ 16) : INT_MAX;
+// Fold the logits z (log2 units) of vocabulary rows vrow, vrow + 8, vrow + 16,
+// vrow + 24 into a running triple.  Rows arrive in increasing order, so only a
+// strictly larger value replaces the argmax.
+__device__ __forceinline__ void fold4(float& m, float& s, int& ix, const float (&z)[4], int vrow) {
+  const float mx = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
+  const int k = z[0] == mx ? 0 : z[1] == mx ? 8 : z[2] == mx ? 16 : 24;
+  const float mn = fmaxf(m, mx);
+  const float add = (fast_exp2(z[0] - mn) + fast_exp2(z[1] - mn)) +
+                    (fast_exp2(z[2] - mn) + fast_exp2(z[3] - mn));
+  s = fmaf(s, fast_exp2(m - mn), add);
+  ix = mx > m ? vrow + k : ix;
+  m = mn;
+}
+
+// Four columns' triples of each thread (index 2 j + e), the same columns in
+// the eight lanes that agree in bits 0 and 1: merge over those lanes; lane l
+// is left with the column j = bit 4, e = bit 3 of l (both values of bit 2 hold
+// it).
+__device__ __forceinline__ void merge_frag8(const float* m, const float* s, const int* ix, int lane,
+                                            float4& out) {
+  const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
+  float am[2], as[2];
+  int ai[2];
 #pragma unroll
-  for (int c = 0; c < 16; ++c) {
-    const float keep = up ? z[c + 16] : z[c];
-    const float send = up ? z[c] : z[c + 16];
-    const float rm = __shfl_xor_sync(0xffffffffu, send, 16);
-    float km = keep, kss = ks;
-    int kii = ki;
-    merge_tri(km, kss, kii, rm, rs, ri);
-    m[c] = km;
-    s[c] = kss;
-    ix[c] = kii;
+  for (int e = 0; e < 2; ++e) {
+    am[e] = up16 ? m[2 + e] : m[e];
+    as[e] = up16 ? s[2 + e] : s[e];
+    ai[e] = up16 ? ix[2 + e] : ix[e];
+    const float rm = __shfl_xor_sync(0xffffffffu, up16 ? m[e] : m[2 + e], 16);
+    const float rs = __shfl_xor_sync(0xffffffffu, up16 ? s[e] : s[2 + e], 16);
+    const int ri = __shfl_xor_sync(0xffffffffu, up16 ? ix[e] : ix[2 + e], 16);
+    merge_tri(am[e], as[e], ai[e], rm, rs, ri);
   }
-#pragma unroll
-  for (int w = 8; w >= 1; w >>= 1) {
-    const bool hi = (lane & w) != 0;
-#pragma unroll
-    for (int c = 0; c < w; ++c) {
-      float km = hi ? m[c + w] : m[c];
-      float kss = hi ? s[c + w] : s[c];
-      int kii = hi ? ix[c + w] : ix[c];
-      const float sm = hi ? m[c] : m[c + w];
-      const float ss = hi ? s[c] : s[c + w];
-      const int si = hi ? ix[c] : ix[c + w];
-      const float rm = __shfl_xor_sync(0xffffffffu, sm, w);
-      const float rss = __shfl_xor_sync(0xffffffffu, ss, w);
-      const int rii = __shfl_xor_sync(0xffffffffu, si, w);
-      merge_tri(km, kss, kii, rm, rss, rii);
-      m[c] = km;
-      s[c] = kss;
-      ix[c] = kii;
-    }
+  float km = up8 ? am[1] : am[0], ks = up8 ? as[1] : as[0];
+  int ki = up8 ? ai[1] : ai[0];
+  {
+    const float rm = __shfl_xor_sync(0xffffffffu, up8 ? am[0] : am[1], 8);
+    const float rs = __shfl_xor_sync(0xffffffffu, up8 ? as[0] : as[1], 8);
+    const int ri = __shfl_xor_sync(0xffffffffu, up8 ? ai[0] : ai[1], 8);
+    merge_tri(km, ks, ki, rm, rs, ri);
   }
-  om = m[0];
-  os = s[0];
-  oi = ix[0];
+  const float rm = __shfl_xor_sync(0xffffffffu, km, 4);
+  const float rs = __shfl_xor_sync(0xffffffffu, ks, 4);
+  const int ri = __shfl_xor_sync(0xffffffffu, ki, 4);
+  merge_tri(km, ks, ki, rm, rs, ri);
+  out = make_float4(km, ks, __int_as_float(ki), 0.0f);
+}
+
+// Fold 32 logits x[k] of one row (times the scale rs, which includes log2 e),
+// vocabulary rows v0 + k, of which the first nvalid exist (the same number in
+// every thread of the warp), into a running triple.  The index is searched for
+// only when the maximum moves, which after the first few chunks it rarely does.
+__device__ __forceinline__ void fold_row32(float& m, float& s, int& ix, const uint32_t (&x)[32],
+                                           float rs, int v0, int nvalid) {
+  float z[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) z[k] = __fmul_rn(__uint_as_float(x[k]), rs);
+  if (nvalid < 32) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) z[k] = k < nvalid ? z[k] : -INFINITY;
+  }
+  float t[4] = {z[0], z[1], z[2], z[3]};
+#pragma unroll
+  for (int k = 4; k < 32; ++k) t[k & 3] = fmaxf(t[k & 3], z[k]);
+  const float cm = fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3]));
+  if (cm > m) {  // strictly: an equal maximum keeps the lower index
+    s *= fast_exp2(m - cm);
+    m = cm;
+    int ci = 0;
+#pragma unroll
+    for (int k = 31; k >= 0; --k) ci = z[k] == cm ? k : ci;
+    ix = v0 + ci;
+  }
+  float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int k = 0; k < 32; ++k) c[k & 3] += fast_exp2(z[k] - m);
+  s += (c[0] + c[1]) + (c[2] + c[3]);
 }
 
 // 32 rows (one per lane) x 32 columns of logits -> lane l holds the
