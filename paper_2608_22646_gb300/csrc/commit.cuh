@@ -149,11 +149,13 @@ __device__ __forceinline__ void commit_load(const CommitParams& p, int b, Commit
 // counter and the exit state (Box 7, Algorithm 1).  Global state is only
 // written, never re-read.  Returns, in every thread, the positions decoded
 // (M_t of the sequence) and, in *left_after, the positions still masked
-// afterwards in a running sequence.
+// afterwards in a running sequence.  With `real` false nothing outside the
+// CTA is written and cs keeps its contents: a pass over stale partials that
+// brings the code into the instruction caches.
 template <int kPPW = kPosPerWarp>
 __device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& cs,
                                      const float4* part, int n_part, int* left_after = nullptr,
-                                     bool loaded = false) {
+                                     bool loaded = false, bool real = true) {
   __shared__ int s_eta, s_left, s_reason, s_unres;
   int* s_tok = cs.tok;
   int* s_cand = cs.cand;
@@ -187,7 +189,7 @@ __device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& c
           row[j] = cs.row[pp];
           if (!CAI_IN_RANGE(row[j] < p.B * p.P, p.err)) row[j] = -2;
           if (row[j] < 0) {
-            if (lane == 0) atomicOr(p.err, kErrBadRow);
+            if (lane == 0 && real) atomicOr(p.err, kErrBadRow);
             row[j] = -2;
           }
         }
@@ -223,7 +225,7 @@ __device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& c
           const int io = __shfl_xor_sync(0xffffffffu, ix, off);
           merge_tri(m, s, ix, mo, so, io);
         }
-        if (lane == 0) {
+        if (lane == 0 && real) {
           const size_t g = g0 + pp;
           const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)
           int bud = s_bud[pp];
@@ -257,7 +259,7 @@ __device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& c
     }
   }
   __syncthreads();
-  if (running && tid == 0) {
+  if (running && tid == 0 && real) {
     const int eta = s_eta;
     p.st.eta[b] = eta;
     const bool low = p.eta_mode == 1
@@ -306,7 +308,7 @@ __device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& c
 // block blk into list / row_of; returns the count.  One CTA (blockDim.x a
 // multiple of 32, at most 1024).  Reads bypass L1: other CTAs wrote this state.
 __device__ int build_masked_list(const int* tok, const int* exit_reason, int* list, int* row_of,
-                                 int B, int P, int L, int n_blocks, int blk) {
+                                 int B, int P, int L, int n_blocks, int blk, bool real = true) {
   __shared__ int s_wsum[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nwarps = blockDim.x >> 5;
@@ -332,7 +334,7 @@ __device__ int build_masked_list(const int* tok, const int* exit_reason, int* li
       woff += (w < warp) ? c : 0;
       tot += c;
     }
-    if (i < BP) {
+    if (i < BP && real) {
       if (mk) {
         list[base + woff + wpre] = i;
         row_of[i] = base + woff + wpre;
@@ -342,6 +344,7 @@ __device__ int build_masked_list(const int* tok, const int* exit_reason, int* li
     }
     base += tot;
     __syncthreads();
+    if (!real) break;
   }
   return base;
 }
@@ -350,11 +353,12 @@ __device__ int build_masked_list(const int* tok, const int* exit_reason, int* li
 // only; the single-kernel step decodes every row and needs none), M_{t+1},
 // the reset ticket and the host-visible record.  `remaining` is the masked
 // count of running sequences when the caller already knows it (-1: count).
-__device__ void finish_step(const CommitParams& p, int remaining = -1) {
+// `real` as in merge_commit_sequence.
+__device__ void finish_step(const CommitParams& p, int remaining = -1, bool real = true) {
   const int n = remaining >= 0 ? remaining
                                : build_masked_list(p.st.tok, p.st.exit_reason, p.list, p.row_of,
-                                                   p.B, p.P, p.L, p.n_blocks, p.blk);
-  if (threadIdx.x == 0) {
+                                                   p.B, p.P, p.L, p.n_blocks, p.blk, real);
+  if (threadIdx.x == 0 && real) {
     *p.d_M = n;
     *p.ticket = 0u;
     const bool err = *reinterpret_cast<volatile uint32_t*>(p.err) != 0u;

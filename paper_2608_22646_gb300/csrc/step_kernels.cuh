@@ -312,29 +312,40 @@ __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const Comm
     M = p.t == 0 ? p.B * p.P : __ldcg(p.d_M);
     commit_load(p, blockIdx.x, cs);
   }
-  grid_dependency_wait();    // partials of this step (and state of the previous one)
-  if (!p.prefetch_state) M = *p.d_M;
-  const bool loaded = p.prefetch_state != 0;
-  if (M >= p.pair_min_M) {
-    const int per_row =
-        pair_partials_per_row(M, p.pair_pairs, pair_swapped(M, p.pair_swap_max_n));
-    if (per_row > 0)
-      merge_commit_sequence<kCommitPPW>(p, blockIdx.x, cs, p.part, per_row, nullptr, loaded);
-    else
-      merge_commit_sequence<kCommitPPW>(p, blockIdx.x, cs, p.rowres, 1, nullptr, loaded);
-  } else {
-    merge_commit_sequence<kCommitPPW>(p, blockIdx.x, cs, p.part, p.n_part, nullptr, loaded);
-  }
-  if (gridDim.x > 1) {
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+  // With prefetch_state the CTA is resident long before the partials are
+  // there: it makes a first pass over whatever the buffers hold, writing
+  // nothing, so that the code (which the step's weight stream has pushed out
+  // of the caches) is there when the second, real pass has to be quick.  From
+  // the partials to the published step: 12.7 -> 7.7 us (4096 x 126464, two
+  // sequences of 33 rows); a step 163 -> 159 us with the LM head's earlier
+  // set-up.
+#pragma unroll 1
+  for (int pass = p.prefetch_state ? 0 : 1; pass < 2; ++pass) {
+    const bool real = pass == 1;
+    if (real) grid_dependency_wait();  // partials of this step (and state of the previous one)
+    if (!p.prefetch_state) M = *p.d_M;
+    const float4* part = p.part;
+    int n_part = p.n_part;
+    if (M >= p.pair_min_M) {
+      n_part = pair_partials_per_row(M, p.pair_pairs, pair_swapped(M, p.pair_swap_max_n));
+      if (n_part == 0) {
+        part = p.rowres;
+        n_part = 1;
+      }
     }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
+    merge_commit_sequence<kCommitPPW>(p, blockIdx.x, cs, part, n_part, nullptr,
+                                      p.prefetch_state != 0, real);
+    if (gridDim.x > 1 && real) {
+      if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+      }
+      __syncthreads();
+      if (!s_last) return;
+      __threadfence();
+    }
+    finish_step(p, -1, real);
   }
-  finish_step(p);
 }
 
 }  // namespace cai
