@@ -226,6 +226,8 @@ struct cai_ctx {
   float norm_eps = 0.0f;
   float* inv_r = nullptr;  // [rows_cap] 1 / sqrt(mean h^2 + eps) of this step's rows
   __nv_bfloat16* h_prev = nullptr;  // [B P, H] previous step's rows (CAI_DIAGNOSTICS)
+  float* drift_ratio = nullptr;     // [B P] and ...
+  unsigned* drift_count = nullptr;  // ... [B]: drift_kernel's scratch
   void (*head_kernel)(CUtensorMap, HeadParams) = nullptr;
   void (*pair_kernel)(CUtensorMap, CUtensorMap, CUtensorMap, PairRowMaps, PairParams) = nullptr;
   int pair_min_M = 0, pair_grid = 0, pair_stages = 0, n_vt = 0, reduce_grid = 0;
@@ -583,6 +585,9 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
     DriftParams dp{};
     dp.hidden = static_cast<const __nv_bfloat16*>(hid);
     dp.prev = c->h_prev;
+    dp.ratio = c->drift_ratio;
+    dp.count = c->drift_count;
+    dp.BP = c->BP;
     dp.drift = c->st.drift;
     dp.P = cfg.P;
     dp.H = cfg.H;
@@ -590,7 +595,9 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
     dp.T = cfg.T;
     dp.blk = c->blk;
     dp.t = t;
-    if (launch_pdl(c->pdl, drift_kernel, cfg.B, kGatherThreads, 0, stream, dp) != cudaSuccess)
+    const int d_grid = (c->BP + kDriftRowsPerCta - 1) / kDriftRowsPerCta;
+    if (launch_pdl(c->pdl, drift_kernel, d_grid, 32 * kDriftRowsPerCta, 0, stream, dp) !=
+        cudaSuccess)
       return check_launch(c);
     c->stats.launches++;
   }
@@ -961,8 +968,16 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   CAI_ALLOC(c->st.run, uint8_t, BL)
   CAI_ALLOC(c->st.stable, int16_t, BL)
   CAI_ALLOC(c->st.drift, float, BN * cfg->T)
-  if (cfg->flags & CAI_DIAGNOSTICS)
+  if (cfg->flags & CAI_DIAGNOSTICS) {
     CAI_ALLOC(c->h_prev, __nv_bfloat16, static_cast<size_t>(c->BP) * cfg->H)
+    CAI_ALLOC(c->drift_ratio, float, c->BP)
+    CAI_ALLOC(c->drift_count, unsigned, cfg->B)
+    if (cudaMemset(c->drift_count, 0, sizeof(unsigned) * cfg->B) != cudaSuccess) {
+      release(c);
+      delete c;
+      return CAI_ERR_CUDA;
+    }
+  }
   CAI_ALLOC(c->list, int, c->BP)
   CAI_ALLOC(c->row_of, int, c->BP)
   CAI_ALLOC(c->d_M, int, 1)

@@ -117,55 +117,77 @@ __global__ void __launch_bounds__(kGatherThreads)
 struct DriftParams {
   const __nv_bfloat16* hidden;  // [B P, H] this step's rows (every position of the block)
   __nv_bfloat16* prev;          // [B P, H] the previous step's rows (kept by this kernel)
+  float* ratio;                 // [B P] relative change of each row
+  unsigned* count;              // [B] rows of a sequence done, zero between launches
   float* drift;                 // [B, n_blocks, T]
-  int P, H, n_blocks, T, blk, t;
+  int BP, P, H, n_blocks, T, blk, t;
 };
 
-// One CTA per sequence: D^(t) = mean over the block's positions of
-// ||h^(t) - h^(t-1)|| / ||h^(t-1)|| (Eq. relative_drift; fp32 sums of the bf16
-// rows), then this step's rows become the previous ones.  At t = 0 only the
-// copy is made.
-__global__ void __launch_bounds__(kGatherThreads) drift_kernel(const DriftParams p) {
-  __shared__ float s_sum[kGatherThreads / 32];
+constexpr int kDriftRowsPerCta = 4;  // one warp per row
+constexpr int kDriftVecs = 8;        // 16-byte loads in flight per lane and operand
+
+// One warp per position: ||h^(t) - h^(t-1)|| / ||h^(t-1)|| (Eq. relative_drift;
+// fp32 sums of the bf16 rows), then this step's row becomes the previous one
+// (at t = 0 only that copy is made).  The warp that finishes a sequence's last
+// row averages the P ratios, in a fixed order, into D^(t).
+//
+// Bound by latency: the rows and their copy are a few MB and mostly in L2.
+// With one CTA per sequence, a warp taking its positions one after the other
+// and one load at a time, a step of 16 sequences of 32 rows of 4096 spent
+// 53 us here.
+__global__ void __launch_bounds__(32 * kDriftRowsPerCta) drift_kernel(const DriftParams p) {
   grid_launch_dependents();  // every thread: the CTA counts once all of them have
   grid_dependency_wait();    // the previous step's drift kernel wrote prev
-  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nw = blockDim.x >> 5, nvec = p.H / 8;
-  float acc = 0.0f;
-  for (int pp = warp; pp < p.P; pp += nw) {
-    const size_t row = static_cast<size_t>(b) * p.P + pp;
-    const uint4* cur = reinterpret_cast<const uint4*>(p.hidden + row * p.H);
-    uint4* prv = reinterpret_cast<uint4*>(p.prev + row * p.H);
-    float num = 0.0f, den = 0.0f;
-    for (int v = lane; v < nvec; v += 32) {
-      const uint4 x = __ldg(cur + v);
-      if (p.t > 0) {
-        const uint4 y = prv[v];
-        const __nv_bfloat16* xe = reinterpret_cast<const __nv_bfloat16*>(&x);
-        const __nv_bfloat16* ye = reinterpret_cast<const __nv_bfloat16*>(&y);
+  const int row = blockIdx.x * kDriftRowsPerCta + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= p.BP) return;
+  const int nvec = p.H / 8;
+  const uint4* cur = reinterpret_cast<const uint4*>(p.hidden + static_cast<size_t>(row) * p.H);
+  uint4* prv = reinterpret_cast<uint4*>(p.prev + static_cast<size_t>(row) * p.H);
+  float num = 0.0f, den = 0.0f;
+  for (int v0 = lane; v0 < nvec; v0 += 32 * kDriftVecs) {
+    uint4 x[kDriftVecs], y[kDriftVecs];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float a = __bfloat162float(ye[i]);
-          const float d = __bfloat162float(xe[i]) - a;
-          num = fmaf(d, d, num);
-          den = fmaf(a, a, den);
-        }
+    for (int j = 0; j < kDriftVecs; ++j) {
+      const int v = v0 + 32 * j;
+      x[j] = v < nvec ? __ldg(cur + v) : make_uint4(0u, 0u, 0u, 0u);
+      y[j] = v < nvec && p.t > 0 ? prv[v] : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < kDriftVecs; ++j) {
+      const __nv_bfloat16* xe = reinterpret_cast<const __nv_bfloat16*>(&x[j]);
+      const __nv_bfloat16* ye = reinterpret_cast<const __nv_bfloat16*>(&y[j]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float a = __bfloat162float(ye[i]);
+        const float d = __bfloat162float(xe[i]) - a;
+        num = fmaf(d, d, num);
+        den = fmaf(a, a, den);
       }
-      prv[v] = x;
+      if (v0 + 32 * j < nvec) prv[v0 + 32 * j] = x[j];
     }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      num += __shfl_xor_sync(0xffffffffu, num, off);
-      den += __shfl_xor_sync(0xffffffffu, den, off);
-    }
-    acc += sqrtf(num) / sqrtf(den);
   }
-  if (lane == 0) s_sum[warp] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0 && p.t > 0) {
-    float tot = 0.0f;
-    for (int w = 0; w < nw; ++w) tot += s_sum[w];
+  if (p.t == 0) return;
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    num += __shfl_xor_sync(0xffffffffu, num, off);
+    den += __shfl_xor_sync(0xffffffffu, den, off);
+  }
+  const int b = row / p.P;
+  unsigned done = 0;
+  if (lane == 0) {
+    p.ratio[row] = sqrtf(num) / sqrtf(den);
+    __threadfence();
+    done = atomicAdd(&p.count[b], 1u);
+  }
+  if (__shfl_sync(0xffffffffu, done, 0) != static_cast<unsigned>(p.P - 1)) return;
+  __threadfence();
+  float tot = 0.0f;
+  for (int pp = lane; pp < p.P; pp += 32) tot += __ldcg(p.ratio + static_cast<size_t>(b) * p.P + pp);
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, off);
+  if (lane == 0) {
     p.drift[(static_cast<size_t>(b) * p.n_blocks + p.blk) * p.T + p.t] = tot / static_cast<float>(p.P);
+    p.count[b] = 0u;
   }
 }
 
