@@ -184,7 +184,7 @@ typedef struct cai_host_state {
 /* Counters kept by the context (host side) since cai_init. */
 typedef struct cai_stats {
   int64_t steps;            /* step calls issued                                   */
-  int64_t launches;         /* kernels launched by this context                    */
+  int64_t launches;         /* kernels launched by this context (resets aside)     */
   int64_t head_launches;    /* launches of the LM-head kernel                      */
   double head_ms;           /* summed device time of profiled LM-head launches     */
   int64_t head_profiled;    /* LM-head launches timed (cai_profile enabled)        */
@@ -325,7 +325,8 @@ int cai_denoise_step(cai_ctx* ctx, const void* hidden, void* stream);
 int cai_block_advance(cai_ctx* ctx, void* stream);
 
 /* Start a new generation with the same weight: every token masked, block 0,
- * counters cleared.  Asynchronous on the stream (device memsets only). */
+ * counters cleared.  Asynchronous on the stream (one kernel, not counted in
+ * cai_stats.launches). */
 int cai_reset(cai_ctx* ctx, void* stream);
 
 /*

@@ -1190,27 +1190,38 @@ int cai_reset(cai_ctx* c, void* stream_v) {
   const cai_config& cfg = c->cfg;
   const size_t BL = static_cast<size_t>(cfg.B) * c->L;
   const size_t BN = static_cast<size_t>(cfg.B) * cfg.n_blocks;
-  bool ok = cudaMemsetAsync(c->st.tok, 0xFF, BL * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.conf, 0, BL * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.s0, 0, BL * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.budget, 0, BL, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.cstep, 0xFF, BL * 2, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.cand, 0xFF, BL * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.ell, 0, cfg.B * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.eta, 0, cfg.B * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.exit_reason, 0, BN * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.exit_step, 0xFF, BN * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.unresolved, 0, BN * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.m_hist, 0, static_cast<size_t>(cfg.n_blocks) * cfg.T * 4, s) ==
-                cudaSuccess &&
-            cudaMemsetAsync(c->st.run, 0, BL, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.stable, 0xFF, BL * 2, s) == cudaSuccess &&
-            cudaMemsetAsync(c->st.drift, 0xFF, BN * cfg.T * 4, s) == cudaSuccess &&  // NaN
-            cudaMemsetAsync(c->ticket, 0, 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->pub, 0, 8, s) == cudaSuccess &&
-            cudaMemsetAsync(c->err, 0, 4, s) == cudaSuccess &&
-            cudaMemsetAsync(c->d_M, 0, 4, s) == cudaSuccess;
-  if (!ok) return fail(c, CAI_ERR_CUDA);
+  ResetParams rp{};
+  unsigned long long most = 0;
+  int n = 0;
+  auto fill = [&](void* ptr, size_t bytes, uint32_t word) {
+    rp.ptr[n] = static_cast<uint4*>(ptr);
+    rp.vecs[n] = (bytes + 15) / 16;
+    rp.word[n] = word;
+    if (rp.vecs[n] > most) most = rp.vecs[n];
+    ++n;
+  };
+  fill(c->st.tok, BL * 4, ~0u);
+  fill(c->st.conf, BL * 4, 0u);
+  fill(c->st.s0, BL * 4, 0u);
+  fill(c->st.budget, BL, 0u);
+  fill(c->st.cstep, BL * 2, ~0u);
+  fill(c->st.cand, BL * 4, ~0u);
+  fill(c->st.ell, cfg.B * 4, 0u);
+  fill(c->st.eta, cfg.B * 4, 0u);
+  fill(c->st.exit_reason, BN * 4, 0u);
+  fill(c->st.exit_step, BN * 4, ~0u);
+  fill(c->st.unresolved, BN * 4, 0u);
+  fill(c->st.m_hist, static_cast<size_t>(cfg.n_blocks) * cfg.T * 4, 0u);
+  fill(c->st.run, BL, 0u);
+  fill(c->st.stable, BL * 2, ~0u);
+  fill(c->st.drift, BN * cfg.T * 4, ~0u);  // NaN
+  fill(c->ticket, 4, 0u);
+  fill(c->pub, 8, 0u);
+  fill(c->err, 4, 0u);
+  fill(c->d_M, 4, 0u);
+  const unsigned long long want = (most + kResetThreads - 1) / kResetThreads;
+  reset_state_kernel<<<static_cast<unsigned>(want < 512 ? want : 512), kResetThreads, 0, s>>>(rp);
+  if (cudaGetLastError() != cudaSuccess) return fail(c, CAI_ERR_CUDA);
   // Step ids keep increasing across resets, so a host-flag write still in
   // flight from the previous generation never satisfies a poll of this one.
   c->blk = 0;

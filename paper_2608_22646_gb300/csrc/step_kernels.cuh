@@ -191,6 +191,30 @@ __global__ void __launch_bounds__(32 * kDriftRowsPerCta) drift_kernel(const Drif
   }
 }
 
+// ----------------------------------------------------------------- reset --
+
+// The state of a new generation: byte-pattern fills of the context's arrays,
+// each rounded up to 16 bytes (every buffer is padded to 256).  One launch
+// instead of a memset per array, whose 19 launches of ~1.5 us each a toy-sized
+// generation spent a tenth of its time on.
+constexpr int kResetFills = 19;
+constexpr int kResetThreads = 256;
+struct ResetParams {
+  uint4* ptr[kResetFills];
+  unsigned long long vecs[kResetFills];  // 16-byte vectors
+  uint32_t word[kResetFills];            // the pattern, 0 or ~0
+};
+
+__global__ void __launch_bounds__(kResetThreads) reset_state_kernel(const ResetParams p) {
+  grid_launch_dependents();  // the first step's weight copies may start; it waits before the state
+  for (int f = 0; f < kResetFills; ++f) {
+    const uint32_t w = p.word[f];
+    for (unsigned long long i = blockIdx.x * static_cast<unsigned long long>(kResetThreads) + threadIdx.x;
+         i < p.vecs[f]; i += static_cast<unsigned long long>(gridDim.x) * kResetThreads)
+      p.ptr[f][i] = make_uint4(w, w, w, w);
+  }
+}
+
 // ------------------------------------------------- bounded-wait test hook --
 
 // Waits, through the same bounded mbar_wait every step kernel uses, on a
