@@ -1322,12 +1322,14 @@ int cai_shard_commit(cai_ctx* c, const void* gathered, int32_t n_shards, void* s
                  stream, mp) != cudaSuccess)
     return check_launch(c);
   c->stats.launches++;
-  // The commit reads the one merged triple per row.
+  // The commit reads the one merged triple per row.  As in a plain step it
+  // reads the state and makes its warming pass before its wait: the last pair
+  // LM head before it in the stream started its dependents after its own wait
+  // for a gather, which ran after this context's previous commit.
   CommitParams cp = commit_params(c, t, step_id);
   cp.part = c->rowres;
   cp.n_part = 1;
   cp.pair_min_M = INT_MAX;
-  cp.prefetch_state = 0;  // the exchange before it is the caller's
   const int commit_threads = c->cfg.P < kCommitThreads / 32 ? 32 * c->cfg.P : kCommitThreads;
   if (launch_pdl(c->pdl, merge_commit_kernel, c->cfg.B, commit_threads, 0, stream, cp) !=
       cudaSuccess)

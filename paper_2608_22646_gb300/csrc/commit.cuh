@@ -209,22 +209,16 @@ __device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& c
       for (int j = 0; j < kPPW; ++j) {
         if (row[j] < 0) continue;  // warp-uniform
         const int pp = base + j * nwarps;
-        float m = kNegBig, s = 0.0f;
-        int ix = INT_MAX;
-#pragma unroll
-        for (int u = 0; u < kPartPerLane; ++u)
-          merge_tri(m, s, ix, q[j][u].x, q[j][u].y, __float_as_int(q[j][u].z));
         for (int k = lane + 32 * kPartPerLane; k < n_part; k += 32) {
           const float4 r = __ldcg(part + static_cast<size_t>(row[j]) * n_part + k);
-          merge_tri(m, s, ix, r.x, r.y, __float_as_int(r.z));
+          int i0 = __float_as_int(q[j][0].z);
+          merge_tri(q[j][0].x, q[j][0].y, i0, r.x, r.y, __float_as_int(r.z));
+          q[j][0].z = __int_as_float(i0);
         }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-          const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-          const float so = __shfl_xor_sync(0xffffffffu, s, off);
-          const int io = __shfl_xor_sync(0xffffffffu, ix, off);
-          merge_tri(m, s, ix, mo, so, io);
-        }
+        __syncwarp();
+        float m, s;
+        int ix;
+        warp_merge(q[j], m, s, ix);
         if (lane == 0 && real) {
           const size_t g = g0 + pp;
           const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)

@@ -728,13 +728,9 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_kernel(const R
       const float4 a = __ldcg(pr + k);
       merge_tri(m, s, ix, a.x, a.y, __float_as_int(a.z));
     }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-      const float so = __shfl_xor_sync(0xffffffffu, s, off);
-      const int io = __shfl_xor_sync(0xffffffffu, ix, off);
-      merge_tri(m, s, ix, mo, so, io);
-    }
+    __syncwarp();
+    const float4 q[1] = {make_float4(m, s, __int_as_float(ix), 0.0f)};
+    warp_merge(q, m, s, ix);
     if (lane == 0) p.rowres[row] = make_float4(m, s, __int_as_float(ix), 0.0f);
   }
 }

@@ -230,6 +230,11 @@ __device__ __forceinline__ void tma_load_2d_pair_nohint(void* dst, const CUtenso
       : "memory");
 }
 
+// Brings the line at p (global memory) into L2.
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory");
+}
+
 // Contiguous bulk copy global -> shared (both 16-byte aligned, size a multiple
 // of 16), completion signalled as transaction bytes on `bar`.
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar,

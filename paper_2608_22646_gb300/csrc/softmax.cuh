@@ -75,6 +75,35 @@ __device__ __forceinline__ void merge_tri(float& m, float& s, int& i, float mo, 
   i = in;
 }
 
+__device__ __forceinline__ float warp_max(float x) {
+  float y;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Merge kN triples of every lane over the whole warp (converged); every lane
+// gets the result, as a sequence of merge_tri would give it up to fp32
+// rounding.  The maximum comes first, in one warp reduction, so that no
+// exponential waits for another: a tree of merge_tri is five of them one
+// after the other.
+template <int kN>
+__device__ __forceinline__ void warp_merge(const float4 (&q)[kN], float& m, float& s, int& ix) {
+  m = q[0].x;
+#pragma unroll
+  for (int u = 1; u < kN; ++u) m = fmaxf(m, q[u].x);
+  m = warp_max(m);
+  s = 0.0f;
+  ix = INT_MAX;
+#pragma unroll
+  for (int u = 0; u < kN; ++u) {
+    s = fmaf(q[u].y, fast_exp2(q[u].x - m), s);
+    ix = q[u].x == m ? min(ix, __float_as_int(q[u].z)) : ix;
+  }
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  ix = __reduce_min_sync(0xffffffffu, ix);
+}
+
 // 32 lanes x 32 columns of online-softmax triples -> lane l holds the merge of
 // column l over the 32 lanes, in m[0], s[0], ix[0].  Five halving steps: at
 // width w each lane keeps half of its live columns and receives the partner's

@@ -49,22 +49,13 @@ __global__ void merge_rows_static_kernel(const float4* part, uint32_t* err, int 
   const bool bad = __ldcg(err) != 0u;
   float m = kNegBig, s = 0.0f;
   int ix = INT_MAX;
-  if (row < M) {
-    float4 q[kStaticMaxParts / 32];  // every load in flight before the first merge
+  if (row < M) {  // the same in the whole warp
+    float4 q[kStaticMaxParts / 32];  // every load in flight before the merge
 #pragma unroll
     for (int u = 0; u < kStaticMaxParts / 32; ++u)
       q[u] = lane + 32 * u < G ? __ldcg(part + static_cast<size_t>(row) * G + lane + 32 * u)
                                : make_float4(kNegBig, 0.0f, __int_as_float(INT_MAX), 0.0f);
-#pragma unroll
-    for (int u = 0; u < kStaticMaxParts / 32; ++u)
-      merge_tri(m, s, ix, q[u].x, q[u].y, __float_as_int(q[u].z));
-  }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-    const float so = __shfl_xor_sync(0xffffffffu, s, off);
-    const int io = __shfl_xor_sync(0xffffffffu, ix, off);
-    merge_tri(m, s, ix, mo, so, io);
+    warp_merge(q, m, s, ix);
   }
   if (lane == 0 && row < M) {
     conf[row] = bad ? __int_as_float(0x7fc00000) : 1.0f / s;

@@ -44,6 +44,16 @@ struct GatherParams {
 __global__ void __launch_bounds__(kGatherThreads)
     gather_rows_kernel(const GatherParams p) {
   grid_launch_dependents();  // every thread: the CTA counts once all of them have
+  if (!p.first && !p.stage_word) {
+    // While the previous step commits: the rows of its list, of which this
+    // step's is a part, towards L2 (the weight has passed through it since).
+    const int q = blockIdx.x * kGatherRowsPerCta + threadIdx.x / 64;
+    const int row = q < p.BP ? __ldcg(p.list + q) : -1;  // stale past the old list
+    if (row >= 0 && row < p.BP) {
+      const char* src = reinterpret_cast<const char*>(p.hidden) + static_cast<size_t>(row) * p.H * 2;
+      for (int o = (threadIdx.x & 63) * 128; o < 2 * p.H; o += 64 * 128) prefetch_l2(src + o);
+    }
+  }
   grid_dependency_wait();  // the previous step's merge wrote list, row_of and d_M
   if (p.stage_word) {
     // The side stream's copy of the rows: one thread waits (bounded) for its
@@ -56,7 +66,10 @@ __global__ void __launch_bounds__(kGatherThreads)
     }
     __syncthreads();
   }
-  const int M = p.first ? p.BP : *p.d_M;
+  // (the row of the list does not wait for M)
+  const int r = blockIdx.x * kGatherRowsPerCta + threadIdx.x / 64;
+  int src_row = p.first || r >= p.BP ? r : __ldcg(p.list + r);
+  const int M = p.first ? p.BP : __ldcg(p.d_M);
   if (p.first) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.BP; i += gridDim.x * blockDim.x) {
       p.list[i] = i;
@@ -65,14 +78,12 @@ __global__ void __launch_bounds__(kGatherThreads)
     if (blockIdx.x == 0 && threadIdx.x == 0) *p.d_M = p.BP;
   }
   const int rows_pad = (M + 15) & ~15;
-  const int r = blockIdx.x * kGatherRowsPerCta + threadIdx.x / 64;
   const int t = threadIdx.x & 63;
   const int nvec = p.H / 8;  // 16-byte vectors per row
   float ss = 0.0f;
   if (r < rows_pad) {
     uint4* dst = reinterpret_cast<uint4*>(p.hc + static_cast<size_t>(r) * p.H);
     if (r < M) {
-      int src_row = p.first ? r : p.list[r];
       if (!CAI_IN_RANGE(src_row >= 0 && src_row < p.BP, p.err)) src_row = 0;
       const uint4* src =
           reinterpret_cast<const uint4*>(p.hidden + static_cast<size_t>(src_row) * p.H);
@@ -283,23 +294,22 @@ __global__ void __launch_bounds__(kShardThreads) shard_rows_kernel(const ShardRo
   for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < p.rows_cap; row += nw) {
     float m = kNegBig, s = 0.0f;
     int ix = INT_MAX;
-    if (row < M) {
-      if (per_row > 0) {
-        for (int k = lane; k < per_row; k += 32) {
-          const float4 a = __ldcg(p.part + static_cast<size_t>(row) * per_row + k);
-          merge_tri(m, s, ix, a.x, a.y, __float_as_int(a.z));
-        }
-      } else if (lane == 0) {
-        const float4 a = __ldcg(p.rowres + row);
-        merge_tri(m, s, ix, a.x, a.y, __float_as_int(a.z));
-      }
+    if (row < M) {  // the same in the whole warp
+      const int n = per_row > 0 ? per_row : 1;
+      const float4* pr = per_row > 0 ? p.part + static_cast<size_t>(row) * per_row : p.rowres + row;
+      float4 q[kPartPerLane];  // every load in flight before the merge
 #pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) {
-        const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-        const float so = __shfl_xor_sync(0xffffffffu, s, off);
-        const int io = __shfl_xor_sync(0xffffffffu, ix, off);
-        merge_tri(m, s, ix, mo, so, io);
+      for (int u = 0; u < kPartPerLane; ++u)
+        q[u] = lane + 32 * u < n ? __ldcg(pr + lane + 32 * u)
+                                 : make_float4(kNegBig, 0.0f, __int_as_float(INT_MAX), 0.0f);
+      for (int k = lane + 32 * kPartPerLane; k < n; k += 32) {
+        const float4 a = __ldcg(pr + k);
+        int i0 = __float_as_int(q[0].z);
+        merge_tri(q[0].x, q[0].y, i0, a.x, a.y, __float_as_int(a.z));
+        q[0].z = __int_as_float(i0);
       }
+      __syncwarp();
+      warp_merge(q, m, s, ix);
     }
     if (lane == 0)
       p.out[row] = make_float4(m, s, __int_as_float(ix == INT_MAX ? INT_MAX : ix + p.v_off), 0.0f);
@@ -327,13 +337,9 @@ __global__ void __launch_bounds__(kShardThreads) shard_merge_kernel(const ShardM
       const float4 a = __ldcg(p.gathered + static_cast<size_t>(k) * p.rows_cap + row);
       merge_tri(m, s, ix, a.x, a.y, __float_as_int(a.z));
     }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-      const float so = __shfl_xor_sync(0xffffffffu, s, off);
-      const int io = __shfl_xor_sync(0xffffffffu, ix, off);
-      merge_tri(m, s, ix, mo, so, io);
-    }
+    __syncwarp();
+    const float4 q[1] = {make_float4(m, s, __int_as_float(ix), 0.0f)};
+    warp_merge(q, m, s, ix);
     if (lane == 0) p.rowres[row] = make_float4(m, s, __int_as_float(ix), 0.0f);
   }
 }
