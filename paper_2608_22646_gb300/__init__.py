@@ -171,6 +171,11 @@ def _ptr(x) -> int | None:
     return x.data_ptr()
 
 
+# Names of the dtypes seen so far (str() of a torch dtype costs more than the
+# rest of the check).
+_DTYPE_NAMES: dict = {}
+
+
 def _buf(x, what: str, dtype: str) -> int | None:
     """Address of a buffer the library reads or writes as a dense array of
     ``dtype`` ("bfloat16", "float32" or "int32"): a tensor or array of that
@@ -185,17 +190,38 @@ def _buf(x, what: str, dtype: str) -> int | None:
             raise ValueError(f"{what}: expected a C-contiguous {np.dtype(want)} array "
                              f"(got {x.dtype}, contiguous={x.flags['C_CONTIGUOUS']})")
         return x.ctypes.data
-    if str(x.dtype) != f"torch.{dtype}" or not x.is_contiguous():
+    dt = x.dtype
+    name = _DTYPE_NAMES.get(dt)
+    if name is None:
+        name = _DTYPE_NAMES[dt] = str(dt).removeprefix("torch.")
+    if name != dtype or not x.is_contiguous():
         raise ValueError(f"{what}: expected a contiguous torch.{dtype} tensor "
                          f"(got {x.dtype}, contiguous={x.is_contiguous()})")
     return x.data_ptr()
 
 
+# PyTorch's functions for the current device and its current stream's handle,
+# once CUDA is known to be there.
+_current_device = _current_raw_stream = None
+
+
 def _stream(s) -> int | None:
+    """Stream handle of ``s``; ``None`` is PyTorch's current stream, asked for
+    at every call.  Building a torch.cuda.Stream to read its handle, after
+    is_available(), took 3.8 us of a step call's 10 (2.5 of them in the
+    library); the raw handle takes 0.2."""
     if s is None:
+        global _current_device, _current_raw_stream
+        if _current_raw_stream is not None:
+            return _current_raw_stream(_current_device())
         import torch
         if torch.cuda.is_available():
-            return torch.cuda.current_stream().cuda_stream
+            handle = torch.cuda.current_stream().cuda_stream  # initialises CUDA
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            dev = getattr(torch._C, "_cuda_getDevice", None)
+            if raw is not None and dev is not None:
+                _current_device, _current_raw_stream = dev, raw
+            return handle
         return None
     if isinstance(s, int):
         return s
