@@ -23,13 +23,13 @@
  * use programmatic dependent launch: each may be scheduled while the kernel
  * before it in the stream still runs, and waits for that kernel to complete
  * before touching anything it produces (setting CAI_PDL=0 in the environment
- * before cai_init launches them plainly instead).  With B P <= 64 a step is
- * one kernel: the LM head over every row of the block, whose last CTA applies
+ * before cai_init launches them plainly instead).  With B P <= 64, or B P <= 128
+ * and a weight of 8 MiB or more, a step is one kernel: the LM head over every row of the block, whose last CTA applies
  * the commit rule; it streams W before the previous step has committed and
  * waits for it only to write its partials and to commit (CAI_FUSED_MAX_BP=n
  * moves the limit, up to 256).  That LM head puts the rows in the MMA's A
  * operand and 256 vocabulary rows in N (up to 128 rows; CAI_ROWS_HEAD=0 uses
- * the swapped-operand kernel instead, W in A and the rows in N).  With B P > 64 a step is gather, LM head,
+ * the swapped-operand kernel instead, W in A and the rows in N).  Otherwise a step is gather, LM head,
  * merge + commit.  The LM head is the CTA-pair
  * kernel (tcgen05 cta_group::2), which picks its orientation per step from
  * the masked-row count M: the rows as MMA N in row tiles of equal width (a
@@ -191,7 +191,7 @@ typedef struct cai_stats {
   int32_t grid;             /* CTAs of the LM-head kernel                          */
   int32_t stages;           /* pipeline stages of the LM-head kernel               */
   int32_t n_max;            /* positions per MMA chunk (N of the swapped MMA)      */
-  int32_t kernels_per_step; /* 1: single-kernel step (B P <= 64); else gather,
+  int32_t kernels_per_step; /* 1: single-kernel step (see above); else gather,
                                LM head(s), row merge if needed, commit (2 to 5)    */
   double step_ms;           /* summed device time of profiled steps, every kernel  */
   int32_t pair_grid;        /* CTAs of the CTA-pair LM head (0: not used)          */

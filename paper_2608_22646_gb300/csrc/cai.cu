@@ -30,11 +30,28 @@ namespace {
 std::atomic<int> g_fail_alloc_after{0};
 std::atomic<int> g_head_grid_limit{0};
 
+// Whether a context of `rows` = B P positions runs single-kernel steps by
+// default.  They decode every row of the block each step and save the gather,
+// the commit kernel and three kernel boundaries; the rows-operand LM head pads
+// the rows to 128 anyway, and the next step's weight stream runs under the
+// commit.  Measured, microseconds a step back to back, single- against
+// multi-kernel with every row masked (multi-kernel at 8 rows in brackets):
+// 96 rows, 4096 x 126464 135 against 159 (152), 1024 x 50003 18.5 against 28.2
+// (21); 128 rows, 144 against 161, 3584 x 152064 145 against 165, 1024 x 22000
+// 18.2 against 21.6 (15); alone 165.8 against 174 at 96 rows and 174.6 against
+// 174.6 at 128.  With a weight of a few MB both are chains of latencies, and
+// above 64 rows the multi-kernel one gets shorter as rows commit (256 x 4096,
+// 128 rows: 15.1 against 15.7, 13.8 at 8 rows).
+constexpr int kFusedMaxRows = 64;       // any weight
+constexpr int kFusedMaxRowsLarge = 128; // weights of at least ...
+constexpr long long kFusedLargeBytes = 8ll << 20;
+bool fused_by_default(int rows, int V, int H) {
+  return rows <= kFusedMaxRows ||
+         (rows <= kFusedMaxRowsLarge && 2ll * V * H >= kFusedLargeBytes);
+}
+
 // Programmatic dependent launch between the step's kernels; CAI_PDL=0 in the
 // environment turns it off (read once per context at cai_init).
-// Largest B P that runs single-kernel steps by default.
-constexpr int kFusedMaxRows = 64;
-
 bool pdl_enabled() {
   const char* e = std::getenv("CAI_PDL");
   return !(e && e[0] == '0');
@@ -52,15 +69,21 @@ bool pair_enabled() {
   return !(e && e[0] == '0');
 }
 
+// CAI_PAIR_SWAP_MAX_N, or 0 when it is not set to a width.
+int pair_swap_env() {
+  const char* n = std::getenv("CAI_PAIR_SWAP_MAX_N");
+  const int v = n ? std::atoi(n) : 0;
+  return v >= 32 && v <= 256 ? v : 0;
+}
+
 // Widest tile the pair kernel runs in the swapped orientation (masked rows in
 // the MMA N dimension, 32-row granularity): CAI_PAIR_SWAP_MAX_N (32..256), or
 // 0 with CAI_PAIR_SWAP=0; default 192.
 int pair_swap_max_n() {
   const char* e = std::getenv("CAI_PAIR_SWAP");
   if (e && e[0] == '0') return 0;
-  const char* n = std::getenv("CAI_PAIR_SWAP_MAX_N");
-  const int v = n ? std::atoi(n) : 0;
-  return v >= 32 && v <= 256 ? v : 192;
+  const int v = pair_swap_env();
+  return v ? v : 192;
 }
 
 // Optional caps on the LM head's W ring depth (CAI_HEAD_STAGES) and tile
@@ -220,6 +243,7 @@ struct cai_ctx {
   int pair_th1 = 0;      // vocabulary rows per CTA and tile of those steps (pair_tile_rows)
   bool use_pair = false; // steps with >= pair_min_M rows run lm_head_pair_kernel
   int swap_max_n = 0;       // ... swapped when its tile width is at most this (pair_swapped)
+  bool swap_on = false;     // the swapped orientation is not turned off (CAI_PAIR_SWAP=0)
   bool head_in_step = true; // the swapped-operand kernel is launched in multi-kernel steps
   bool need_reduce = false; // some step size leaves per-tile partials to reduce_partials_kernel
   bool norm = false;     // the model's final RMSNorm is part of the head (cai_init_rmsnorm)
@@ -385,8 +409,8 @@ double pos_factor_of(const cai_config& c, int p) {
 // theta_i(t) of position p in block b1 (1-based), Eq. position_threshold:
 // the block's threshold times the position factor, clipped, in double, then
 // rounded once to the fp32 value the commit rule compares against.
-float theta_token_of(const cai_config& c, int b1, int t, int p) {
-  double th = theta_block_of(c, b1, t) * pos_factor_of(c, p);
+float theta_token_of(const cai_config& c, double theta_block, int p) {
+  double th = theta_block * pos_factor_of(c, p);
   th = th < c.clip_lo ? c.clip_lo : th;
   th = th > c.clip_hi ? c.clip_hi : th;
   return static_cast<float>(th);
@@ -430,7 +454,8 @@ CommitParams commit_params(cai_ctx* c, int t, int64_t step_id) {
   cp.budget_half = (cfg.flags & CAI_QUARTER_POS) ? cfg.P / 2 : 32;
   cp.budget_late = (cfg.flags & CAI_QUARTER_POS) ? 3 * cfg.P / 4 : 48;
   cp.flags = cfg.flags;
-  for (int p = 0; p < cfg.P; ++p) cp.theta_tab[p] = theta_token_of(cfg, c->blk + 1, t, p);
+  const double theta_block = theta_block_of(cfg, c->blk + 1, t);
+  for (int p = 0; p < cfg.P; ++p) cp.theta_tab[p] = theta_token_of(cfg, theta_block, p);
   return cp;
 }
 
@@ -657,7 +682,7 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
   if (c->head_in_step) {
     const CUtensorMap& tm_rows =
         !c->fused ? c->tm_h : stage_slot >= 0 ? c->tm_stage[stage_slot] : c->tm_hid;
-    if (launch_pdl(c->pdl, c->head_kernel, c->G, kHeadThreads, c->head_smem, stream, tm_rows,
+    if (launch_pdl(c->pdl, c->head_kernel, c->G, c->rows_head ? kRowsThreads : kHeadThreads, c->head_smem, stream, tm_rows,
                    hp) != cudaSuccess)
       return check_launch(c);
     c->stats.launches++;
@@ -765,15 +790,11 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   c->rows_cap = round_up(c->BP, 16);
   c->pdl = pdl_enabled();
   c->nvtx = nvtx_enabled();
-  // Single-kernel steps decode every row of the block each step (the
-  // rows-operand LM head pads the rows to 128 anyway) and save the gather and
-  // commit launches; larger batches run multi-kernel steps, whose pair kernel
-  // decodes only the masked rows.  Measured, LLaDA shape, positions/s,
-  // single- against multi-kernel: B P = 64 197.8k against 169.5k, B P = 128
-  // 329.3k against 331.5k.  CAI_FUSED_MAX_BP overrides the limit (up to 256;
+  // CAI_FUSED_MAX_BP overrides the limit of single-kernel steps (up to 256;
   // above 128 rows the swapped-operand kernel runs).
   const int fmax = env_int("CAI_FUSED_MAX_BP");
-  c->fused = !shard && c->BP <= (fmax > 0 && fmax <= kChunkN ? fmax : kFusedMaxRows);
+  c->fused = !shard && (fmax > 0 && fmax <= kChunkN ? c->BP <= fmax
+                                                     : fused_by_default(c->BP, cfg->V, cfg->H));
   c->norm = g != nullptr;
   c->norm_eps = static_cast<float>(eps);
   c->head_kernel = c->norm ? lm_head_softmax_kernel<true> : lm_head_softmax_kernel<false>;
@@ -785,6 +806,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   c->use_pair = shard || (!c->fused && pair_enabled());
   c->swap_max_n = c->use_pair ? pair_swap_max_n() : 0;
   if (shard && c->swap_max_n < kSwapColStep) c->swap_max_n = 192;
+  c->stats.pair_swap_max_n = c->swap_max_n;
+  c->swap_on = c->swap_max_n > 0;
   c->pair_kernel = c->norm ? lm_head_pair_kernel<true> : lm_head_pair_kernel<false>;
 
   // LM-head launch shape.  N chunk (positions per MMA), grid (one CTA per SM,
@@ -799,7 +822,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   // the W stream it rides on), and the swapped-operand kernel is not launched.
   if (c->use_pair) {
     const int mset = env_int("CAI_PAIR_MIN_M");
-    c->pair_min_M = mset > 0 ? mset : (c->swap_max_n >= kSwapColStep ? 1 : 32);
+    c->pair_min_M = mset > 0 ? mset : (c->swap_on ? 1 : 32);
   }
   c->head_in_step = !c->use_pair || c->pair_min_M > 1;
   c->n_max = c->rows_cap < kChunkN ? c->rows_cap : kChunkN;
@@ -1146,7 +1169,6 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   c->stats.stages = c->n_stages;
   c->stats.n_max = c->n_max;
   c->stats.pair_grid = c->use_pair ? c->pair_grid : 0;
-  c->stats.pair_swap_max_n = c->swap_max_n;
   c->stats.pair_stages = c->use_pair ? c->pair_stages : 0;
   c->stats.head_rows = c->rows_head ? 1 : 0;
   c->stats.kernels_per_step =
@@ -1591,7 +1613,8 @@ int cai_test_theta_table(const cai_config* cfg, int32_t blk, int32_t t, float* o
   const int r = validate(cfg);
   if (r != CAI_OK) return r;
   if (blk < 0 || blk >= cfg->n_blocks || t < 0 || t >= cfg->T) return CAI_ERR_ARG;
-  for (int p = 0; p < cfg->P; ++p) out[p] = theta_token_of(*cfg, blk + 1, t, p);
+  const double theta_block = theta_block_of(*cfg, blk + 1, t);
+  for (int p = 0; p < cfg->P; ++p) out[p] = theta_token_of(*cfg, theta_block, p);
   return CAI_OK;
 }
 

@@ -96,8 +96,9 @@ __device__ __forceinline__ int budget_tier(float s, int p, int half, int late) {
   return 32;
 }
 
-// Per-position working set of merge_commit_sequence, in shared memory the
-// caller provides (the LM-head kernel lends its drained W ring).
+// Working set of one commit, in shared memory the caller provides (the LM-head
+// kernel lends its drained W ring): the block's positions of one or several
+// sequences, at most kMaxP of them, sequence by sequence.
 struct CommitSmem {
   int tok[kMaxP];      // token after this step (kMask while masked)
   int cand[kMaxP];     // argmax of the previous decoded step, then of this step
@@ -106,196 +107,191 @@ struct CommitSmem {
   uint8_t bud[kMaxP];  // budget before this step
   uint8_t run[kMaxP];  // diagnostics: same-argmax run before this step
   int16_t stable[kMaxP];  // diagnostics: stability step before this step
-  int running;         // the sequence has not left the block
-  int ell;             // low-yield counter before this step
+  // per sequence
+  int running[kMaxP];  // the sequence has not left the block
+  int ell[kMaxP];      // low-yield counter before this step
+  int eta[kMaxP], left[kMaxP], unres[kMaxP], reason[kMaxP];  // this step's counts and exit
+  int decoded, remaining;  // over all sequences: rows decoded, rows still masked afterwards
 };
 
-// Reads what one step of Algorithm 1 needs of sequence b's state into cs, in
-// one round of loads by the whole calling CTA (visible to it after its next
-// __syncthreads): the block's tokens and budgets, the exit state, ell, and
-// the partial row of every position.  All of it was written by the previous
-// step's commit (or by the reset) except, at a block's first step, the row
-// list, which the gather then makes the identity; so a commit that follows an
-// LM head which itself waited for the previous step may read it before
-// waiting for the partials.
-__device__ __forceinline__ void commit_load(const CommitParams& p, int b, CommitSmem& cs) {
+// Reads what one step of Algorithm 1 needs of the state of sequences [b0, b0 +
+// nb) into cs, in one round of loads by the whole calling CTA (visible to it
+// after its next __syncthreads): the block's tokens and budgets, the exit
+// state, ell, and the partial row of every position.  All of it was written by
+// the previous step's commit (or by the reset) except, at a block's first step,
+// the row list, which the gather then makes the identity; so a commit that
+// follows an LM head which itself waited for the previous step may read it
+// before waiting for the partials.
+__device__ __forceinline__ void commit_load(const CommitParams& p, int b0, int nb, CommitSmem& cs) {
   const int tid = threadIdx.x;
-  const int eb = b * p.n_blocks + p.blk;
-  const size_t g0 = static_cast<size_t>(b) * p.L + p.blk * p.P;
-  if (tid == 0) {
-    cs.running = __ldcg(&p.st.exit_reason[eb]) == kRunning;
-    cs.ell = __ldcg(&p.st.ell[b]);
+  for (int q = tid; q < nb; q += blockDim.x) {
+    cs.running[q] = __ldcg(&p.st.exit_reason[(b0 + q) * p.n_blocks + p.blk]) == kRunning;
+    cs.ell[q] = __ldcg(&p.st.ell[b0 + q]);
+    cs.eta[q] = cs.left[q] = cs.unres[q] = 0;
+    cs.reason[q] = kRunning;
   }
+  if (tid == 0) cs.decoded = cs.remaining = 0;
   const bool diag = (p.flags & kFlagDiag) != 0;
   const bool ident = p.identity_rows || p.t == 0;
-  for (int pp = tid; pp < p.P; pp += blockDim.x) {
-    cs.tok[pp] = __ldcg(&p.st.tok[g0 + pp]);
-    cs.bud[pp] = p.st.budget[g0 + pp];
-    cs.row[pp] = ident ? b * p.P + pp : __ldcg(&p.row_of[b * p.P + pp]);
+  for (int i = tid; i < nb * p.P; i += blockDim.x) {
+    const int q = i / p.P;
+    const size_t g = static_cast<size_t>(b0 + q) * p.L + p.blk * p.P + (i - q * p.P);
+    cs.tok[i] = __ldcg(&p.st.tok[g]);
+    cs.bud[i] = p.st.budget[g];
+    cs.row[i] = ident ? b0 * p.P + i : __ldcg(&p.row_of[b0 * p.P + i]);
     if (diag) {
-      cs.cand[pp] = __ldcg(&p.st.cand[g0 + pp]);
-      cs.run[pp] = __ldcg(&p.st.run[g0 + pp]);
-      cs.stable[pp] = __ldcg(&p.st.stable[g0 + pp]);
+      cs.cand[i] = __ldcg(&p.st.cand[g]);
+      cs.run[i] = __ldcg(&p.st.run[g]);
+      cs.stable[i] = __ldcg(&p.st.stable[g]);
     }
   }
 }
 
-// One step of Algorithm 1 for sequence b, by the whole calling CTA (blockDim.x
-// a multiple of 32; every thread must call it).  The sequence's state is in
-// cs (commit_load, by this call unless `loaded`); warps merge the partials of
-// the still-masked positions (kPPW at a time, all loads issued before any
-// merge) and lane 0 applies the commit rule (Box 6, Eq. position_commit,
-// with the step-zero init of Boxes 2 and 5); thread 0 updates the low-yield
-// counter and the exit state (Box 7, Algorithm 1).  Global state is only
-// written, never re-read.  Returns, in every thread, the positions decoded
-// (M_t of the sequence) and, in *left_after, the positions still masked
-// afterwards in a running sequence.  With `real` false nothing outside the
-// CTA is written and cs keeps its contents: a pass over stale partials that
-// brings the code into the instruction caches.
+// One step of Algorithm 1 for the sequences [b0, b0 + nb) that commit_load has
+// read into cs (nb P <= kMaxP), by the whole calling CTA (blockDim.x a multiple
+// of 32; every thread must call it).  Warps merge the partials of the
+// still-masked positions (kPPW at a time, all loads issued before any merge)
+// and lane 0 applies the commit rule (Box 6, Eq. position_commit, with the
+// step-zero init of Boxes 2 and 5); one thread per sequence updates the
+// low-yield counter and the exit state (Box 7, Algorithm 1).  Global state is
+// only written, never re-read.  Leaves in cs, for every thread, the positions
+// decoded and those still masked afterwards in running sequences.  With `real`
+// false nothing outside the CTA is written and cs keeps its contents: a pass
+// over stale partials that brings the code into the instruction caches.
 template <int kPPW = kPosPerWarp>
-__device__ int merge_commit_sequence(const CommitParams& p, int b, CommitSmem& cs,
-                                     const float4* part, int n_part, int* left_after = nullptr,
-                                     bool loaded = false, bool real = true) {
-  __shared__ int s_eta, s_left, s_reason, s_unres;
-  int* s_tok = cs.tok;
-  int* s_cand = cs.cand;
-  float* s_conf = cs.conf;
-  uint8_t* s_bud = cs.bud;
+__device__ void merge_commit(const CommitParams& p, int b0, int nb, CommitSmem& cs,
+                             const float4* part, int n_part, bool real = true) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nwarps = blockDim.x >> 5;
-  const int eb = b * p.n_blocks + p.blk;
-  const size_t g0 = static_cast<size_t>(b) * p.L + p.blk * p.P;
-  if (!loaded) commit_load(p, b, cs);
-  if (tid == 0) {
-    s_eta = 0;
-    s_left = 0;
-    s_reason = kRunning;
-    s_unres = 0;
-  }
+  const int n = nb * p.P;
   const bool diag = (p.flags & kFlagDiag) != 0;
-  __syncthreads();
-  const bool running = cs.running != 0;
   const bool gating = (p.flags & kFlagGating) != 0;
+  __syncthreads();
 
-  if (running) {
-    for (int base = warp; base < p.P; base += nwarps * kPPW) {
-      int row[kPPW];
-      float4 q[kPPW][kPartPerLane];
+  for (int base = warp; base < n; base += nwarps * kPPW) {
+    int row[kPPW];
+    float4 q[kPPW][kPartPerLane];
 #pragma unroll
-      for (int j = 0; j < kPPW; ++j) {
-        const int pp = base + j * nwarps;
-        row[j] = -1;
-        if (pp < p.P && s_tok[pp] == kMask) {
-          row[j] = cs.row[pp];
-          if (!CAI_IN_RANGE(row[j] < p.B * p.P, p.err)) row[j] = -2;
-          if (row[j] < 0) {
-            if (lane == 0 && real) atomicOr(p.err, kErrBadRow);
-            row[j] = -2;
-          }
+    for (int j = 0; j < kPPW; ++j) {
+      const int i = base + j * nwarps;
+      row[j] = -1;
+      if (i < n && cs.tok[i] == kMask && cs.running[i / p.P]) {
+        row[j] = cs.row[i];
+        if (!CAI_IN_RANGE(row[j] < p.B * p.P, p.err)) row[j] = -2;
+        if (row[j] < 0) {
+          if (lane == 0 && real) atomicOr(p.err, kErrBadRow);
+          row[j] = -2;
         }
       }
+    }
 #pragma unroll
-      for (int j = 0; j < kPPW; ++j) {
-        const float4* pr = part + static_cast<size_t>(row[j] < 0 ? 0 : row[j]) * n_part;
+    for (int j = 0; j < kPPW; ++j) {
+      const float4* pr = part + static_cast<size_t>(row[j] < 0 ? 0 : row[j]) * n_part;
 #pragma unroll
-        for (int u = 0; u < kPartPerLane; ++u) {
-          const int k = lane + 32 * u;
-          q[j][u] = (row[j] >= 0 && k < n_part)
-                        ? __ldcg(pr + k)
-                        : make_float4(kNegBig, 0.0f, __int_as_float(INT_MAX), 0.0f);
-        }
+      for (int u = 0; u < kPartPerLane; ++u) {
+        const int k = lane + 32 * u;
+        q[j][u] = (row[j] >= 0 && k < n_part)
+                      ? __ldcg(pr + k)
+                      : make_float4(kNegBig, 0.0f, __int_as_float(INT_MAX), 0.0f);
       }
+    }
 #pragma unroll
-      for (int j = 0; j < kPPW; ++j) {
-        if (row[j] < 0) continue;  // warp-uniform
-        const int pp = base + j * nwarps;
-        for (int k = lane + 32 * kPartPerLane; k < n_part; k += 32) {
-          const float4 r = __ldcg(part + static_cast<size_t>(row[j]) * n_part + k);
-          int i0 = __float_as_int(q[j][0].z);
-          merge_tri(q[j][0].x, q[j][0].y, i0, r.x, r.y, __float_as_int(r.z));
-          q[j][0].z = __int_as_float(i0);
+    for (int j = 0; j < kPPW; ++j) {
+      if (row[j] < 0) continue;  // warp-uniform
+      const int i = base + j * nwarps;
+      for (int k = lane + 32 * kPartPerLane; k < n_part; k += 32) {
+        const float4 r = __ldcg(part + static_cast<size_t>(row[j]) * n_part + k);
+        int i0 = __float_as_int(q[j][0].z);
+        merge_tri(q[j][0].x, q[j][0].y, i0, r.x, r.y, __float_as_int(r.z));
+        q[j][0].z = __int_as_float(i0);
+      }
+      __syncwarp();
+      float m, s;
+      int ix;
+      warp_merge(q[j], m, s, ix);
+      if (lane == 0 && real) {
+        const int sq = i / p.P, pp = i - sq * p.P;
+        const size_t g = static_cast<size_t>(b0 + sq) * p.L + p.blk * p.P + pp;
+        const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)
+        int bud = cs.bud[i];
+        if (p.t == 0) {
+          bud = budget_tier(c, pp, p.budget_half, p.budget_late);
+          p.st.s0[g] = c;
+          p.st.budget[g] = static_cast<uint8_t>(bud);
         }
-        __syncwarp();
-        float m, s;
-        int ix;
-        warp_merge(q[j], m, s, ix);
-        if (lane == 0 && real) {
-          const size_t g = g0 + pp;
-          const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)
-          int bud = s_bud[pp];
-          if (p.t == 0) {
-            bud = budget_tier(c, pp, p.budget_half, p.budget_late);
-            p.st.s0[g] = c;
-            p.st.budget[g] = static_cast<uint8_t>(bud);
-          }
-          if (diag) {
-            // Section 2.1: stable once the argmax has held for three decoded steps.
-            const int run = (p.t > 0 && s_cand[pp] == ix) ? cs.run[pp] + 1 : 1;
-            p.st.run[g] = static_cast<uint8_t>(run < 255 ? run : 255);
-            if (run >= 3 && cs.stable[pp] < 0) p.st.stable[g] = static_cast<int16_t>(p.t);
-          }
-          p.st.conf[g] = c;
-          p.st.cand[g] = ix;
-          s_conf[pp] = c;
-          s_cand[pp] = ix;
-          const bool by_conf = c >= p.theta_tab[pp];
-          const bool by_budget = gating && p.t >= bud;
-          if (by_conf || by_budget) {
-            s_tok[pp] = ix;
-            p.st.tok[g] = ix;
-            p.st.cstep[g] = static_cast<int16_t>(p.t);
-            atomicAdd(&s_eta, 1);
-          } else {
-            atomicAdd(&s_left, 1);
-          }
+        if (diag) {
+          // Section 2.1: stable once the argmax has held for three decoded steps.
+          const int run = (p.t > 0 && cs.cand[i] == ix) ? cs.run[i] + 1 : 1;
+          p.st.run[g] = static_cast<uint8_t>(run < 255 ? run : 255);
+          if (run >= 3 && cs.stable[i] < 0) p.st.stable[g] = static_cast<int16_t>(p.t);
+        }
+        p.st.conf[g] = c;
+        p.st.cand[g] = ix;
+        cs.conf[i] = c;
+        cs.cand[i] = ix;
+        const bool by_conf = c >= p.theta_tab[pp];
+        const bool by_budget = gating && p.t >= bud;
+        if (by_conf || by_budget) {
+          cs.tok[i] = ix;
+          p.st.tok[g] = ix;
+          p.st.cstep[g] = static_cast<int16_t>(p.t);
+          atomicAdd(&cs.eta[sq], 1);
+        } else {
+          atomicAdd(&cs.left[sq], 1);
         }
       }
     }
   }
   __syncthreads();
-  if (running && tid == 0 && real) {
-    const int eta = s_eta;
-    p.st.eta[b] = eta;
+  if (!real) return;
+  bool exits = false;
+  for (int q = tid; q < nb; q += blockDim.x) {
+    if (!cs.running[q]) continue;
+    const int eta = cs.eta[q];
+    p.st.eta[b0 + q] = eta;
     const bool low = p.eta_mode == 1
                          ? (static_cast<double>(eta) / (static_cast<double>(p.n_blocks) * p.P) <
                             static_cast<double>(p.eta_bar))
                          : (static_cast<float>(eta) < p.eta_bar);
     // Algorithm 1 sets ell <- 0 before the block's first step.
-    const int ell = low ? (p.t == 0 ? 0 : cs.ell) + 1 : 0;
-    p.st.ell[b] = ell;
+    const int ell = low ? (p.t == 0 ? 0 : cs.ell[q]) + 1 : 0;
+    p.st.ell[b0 + q] = ell;
     int reason = kRunning;
     if (gating && ell >= p.K)
       reason = kExitGrind;
-    else if (s_left == 0)
+    else if (cs.left[q] == 0)
       reason = kExitDone;
     else if (p.t == p.T - 1)
       reason = kExitTmax;
-    s_reason = reason;
+    cs.reason[q] = reason;
+    atomicAdd(&cs.decoded, eta + cs.left[q]);
+    if (reason == kRunning)
+      atomicAdd(&cs.remaining, cs.left[q]);
+    else
+      exits = true;
   }
-  __syncthreads();
-  const int reason = s_reason;
-  const int decoded = s_eta + s_left;
-  if (running && reason != kRunning) {
-    for (int pp = tid; pp < p.P; pp += blockDim.x) {
-      if (s_tok[pp] != kMask) continue;
-      const size_t g = g0 + pp;
-      if ((reason == kExitGrind && s_conf[pp] > p.theta_fb) || (p.flags & kFlagFlush)) {
-        p.st.tok[g] = s_cand[pp];
-        p.st.cstep[g] = static_cast<int16_t>(p.t);
-      } else {
-        atomicAdd(&s_unres, 1);
-      }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      p.st.exit_reason[eb] = reason;
-      p.st.exit_step[eb] = p.t;
-      p.st.unresolved[eb] = s_unres;
+  if (!__syncthreads_or(exits)) return;
+  for (int i = tid; i < n; i += blockDim.x) {
+    const int sq = i / p.P;
+    const int reason = cs.reason[sq];
+    if (reason == kRunning || cs.tok[i] != kMask) continue;
+    const size_t g = static_cast<size_t>(b0 + sq) * p.L + p.blk * p.P + (i - sq * p.P);
+    if ((reason == kExitGrind && cs.conf[i] > p.theta_fb) || (p.flags & kFlagFlush)) {
+      p.st.tok[g] = cs.cand[i];
+      p.st.cstep[g] = static_cast<int16_t>(p.t);
+    } else {
+      atomicAdd(&cs.unres[sq], 1);
     }
   }
-  if (left_after) *left_after = (running && reason == kRunning) ? s_left : 0;
   __syncthreads();
-  return decoded;
+  for (int q = tid; q < nb; q += blockDim.x) {
+    if (cs.reason[q] == kRunning) continue;
+    const int eb = (b0 + q) * p.n_blocks + p.blk;
+    p.st.exit_reason[eb] = cs.reason[q];
+    p.st.exit_step[eb] = p.t;
+    p.st.unresolved[eb] = cs.unres[q];
+  }
+  __syncthreads();
 }
 
 // Compact, in (b, p) order, the still-masked tokens of running sequences of
@@ -347,7 +343,7 @@ __device__ int build_masked_list(const int* tok, const int* exit_reason, int* li
 // only; the single-kernel step decodes every row and needs none), M_{t+1},
 // the reset ticket and the host-visible record.  `remaining` is the masked
 // count of running sequences when the caller already knows it (-1: count).
-// `real` as in merge_commit_sequence.
+// `real` as in merge_commit.
 __device__ void finish_step(const CommitParams& p, int remaining = -1, bool real = true) {
   const int n = remaining >= 0 ? remaining
                                : build_masked_list(p.st.tok, p.st.exit_reason, p.list, p.row_of,

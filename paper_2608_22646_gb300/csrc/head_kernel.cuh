@@ -303,15 +303,11 @@ __device__ __forceinline__ void fused_step_commit(const CommitParams& cp, uint8_
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  int decoded = 0, remaining = 0;
-  for (int b = 0; b < cp.B; ++b) {
-    int left = 0;
-    decoded += merge_commit_sequence(cp, b, *reinterpret_cast<CommitSmem*>(free_smem), cp.part,
-                                     cp.n_part, &left);
-    remaining += left;
-  }
-  if (threadIdx.x == 0) *cp.m_hist_slot = decoded;
-  finish_step(cp, remaining);
+  CommitSmem& cs = *reinterpret_cast<CommitSmem*>(free_smem);
+  commit_load(cp, 0, cp.B, cs);
+  merge_commit(cp, 0, cp.B, cs, cp.part, cp.n_part);
+  if (threadIdx.x == 0) *cp.m_hist_slot = cs.decoded;
+  finish_step(cp, cs.remaining);
 }
 
 // ---------------------------------------------------------------- kernel --
@@ -565,7 +561,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
     if constexpr (kNorm) {
       __shared__ float s_scale[kChunkN];
       if (p.fused) {
-        epilogue_row_scales(p.hid, M, p.H, p.norm_eps, s_scale, ew, lane);
+        epilogue_row_scales<4>(p.hid, M, p.H, p.norm_eps, s_scale, ew, lane);
         scale = s_scale;
       }
     }

@@ -38,12 +38,12 @@
 // one (see the pair kernel): alone, LLaDA's 32 rows 160.6 -> 159.6 us and 64
 // rows 168.4 -> 166.6 us; back to back 1.5 % of a generation.
 //
-// Roles (192 threads): warp 0 producer (W stages by bulk copy, row stages by
-// TMA); warp 1 allocates tensor memory and issues the MMAs; warps 2..5
+// Roles (320 threads): warp 0 producer (W stages by bulk copy, row stages by
+// TMA); warp 1 allocates tensor memory and issues the MMAs; warps 2..9
 // epilogue: tensor-memory lane r holds row r's logits, so
-// the thread of lane r runs a serial online softmax over the group's columns
-// (only warps whose 32 lanes hold rows < M have work).  Each thread writes
-// one partial per (row, CTA); the last CTA merges them and commits the step
+// two threads (half of the columns each) run a serial online softmax over the
+// group's columns (only warps whose 32 lanes hold rows < M have work).  One of
+// them writes one partial per (row, CTA); the last CTA merges them and commits the step
 // (fused_step_commit), as in the single-kernel step of
 // lm_head_softmax_kernel, with the same cross-step behaviour under
 // programmatic dependent launch.
@@ -61,6 +61,8 @@ constexpr int kRowsGroupRows = 256;                  // MMA N: vocabulary rows p
 constexpr int kRowsWStage = kRowsGroupRows * 128;    // 32 KiB: one K block of a group
 constexpr int kRowsHStageMax = kRowsM * 128;         // 16 KiB: all 128 rows of a K block
 constexpr int kRowsTmemCols = 2 * kRowsGroupRows;    // two accumulators
+constexpr int kRowsEpiWarps = 8;                     // two per tensor-memory quarter
+constexpr int kRowsThreads = 64 + 32 * kRowsEpiWarps;
 
 // Bytes between two rows stages for a step of M rows (see above).
 __host__ __device__ inline int rows_h_stride(int M) {
@@ -72,7 +74,7 @@ __host__ __device__ inline int rows_h_stride(int M) {
 __host__ __device__ inline size_t rows_smem_bytes(int n_stages, int n_bslots, int h_stride) {
   return 1024 + static_cast<size_t>(n_bslots) * h_stride +
          static_cast<size_t>(n_stages) * kRowsWStage +
-         static_cast<size_t>(2 * n_stages + 2 * n_bslots + 5) * 8 + 16;
+         static_cast<size_t>(2 * n_stages + 2 * n_bslots + 6) * 8 + 16;
 }
 
 struct RowsSmem {
@@ -83,8 +85,9 @@ struct RowsSmem {
   uint64_t* full_h;   // n_bslots
   uint64_t* empty_h;  // n_bslots
   uint64_t* accf;     // 2: accumulator ready
-  uint64_t* acce;     // 2: accumulator drained by the four epilogue warps
+  uint64_t* acce;     // 2: accumulator drained by the epilogue warps
   uint64_t* drain;    // 1
+  uint64_t* xch;      // 1: the second half's epilogue warps wrote their triples
   uint32_t* tmem_slot;
   volatile int* abort;
   volatile int* skip;
@@ -104,7 +107,8 @@ __device__ __forceinline__ RowsSmem rows_carve(uint8_t* raw, int n_stages, int n
   s.accf = s.empty_h + n_bslots;
   s.acce = s.accf + 2;
   s.drain = s.acce + 2;
-  s.tmem_slot = reinterpret_cast<uint32_t*>(s.drain + 1);
+  s.xch = s.drain + 1;
+  s.tmem_slot = reinterpret_cast<uint32_t*>(s.xch + 1);
   s.abort = reinterpret_cast<volatile int*>(s.tmem_slot + 1);
   s.skip = s.abort + 1;
   return s;
@@ -185,7 +189,7 @@ __global__ void pack_weight_rows_kernel(const uint4* __restrict__ W, uint4* __re
 // r's logits are scaled by 1 / sqrt(mean h^2 + eps) of the row, which the
 // epilogue warps compute from the step's rows (p.hid).
 template <bool kNorm>
-__global__ void __launch_bounds__(kHeadThreads, 1)
+__global__ void __launch_bounds__(kRowsThreads, 1)
     lm_head_rows_kernel(const __grid_constant__ CUtensorMap tm_h, const HeadParams p) {
   extern __shared__ uint8_t smem_raw[];
   const int warp = threadIdx.x >> 5;
@@ -211,9 +215,10 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&sm.accf[a], 1);
-      mbar_init(&sm.acce[a], 4);
+      mbar_init(&sm.acce[a], kRowsEpiWarps);
     }
     mbar_init(sm.drain, 1);
+    mbar_init(sm.xch, kRowsEpiWarps / 2);
     *sm.abort = 0;
     *sm.skip = 0;
     fence_mbar_init();
@@ -375,6 +380,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
   } else {
     // --------------------------------------------------------- epilogue --
     const int quarter = warp & 3;  // tensor-memory lanes 32 quarter .. 32 quarter + 31
+    const int hf = (warp - 2) >> 2;  // half of a group's 32-column chunks
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const int row = quarter * 32 + lane;
     const bool active = quarter * 32 < M;  // warp-uniform: some lane holds a row
@@ -386,7 +392,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
       // group accumulates.  Nothing here depends on an earlier kernel, so the
       // accumulators are drained as in a step without the norm.
       __shared__ float s_scale[kRowsM];
-      epilogue_row_scales(p.hid, M, p.H, p.norm_eps, s_scale, warp - 2, lane);
+      epilogue_row_scales<kRowsEpiWarps>(p.hid, M, p.H, p.norm_eps, s_scale, warp - 2, lane);
       if (row < M) rs = kLog2e * s_scale[row];
     }
     Ring racc;
@@ -406,38 +412,16 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
         const uint32_t tbase =
             tmem_base + lane_base + static_cast<uint32_t>(racc.slot * kRowsGroupRows);
         const int vbase = pl.group_row0(g);
-        const int gr = pl.group_rows(g);
-        const int nch = (gr + 31) >> 5;
+        // Vocabulary rows past the group's (stale stage bytes) or past V are left out.
+        const int nrow = min(pl.group_rows(g), p.V - vbase);
+        const int nch = (pl.group_rows(g) + 31) >> 5;
+        const int c1 = hf ? nch : (nch + 1) >> 1;
 #pragma unroll 1
-        for (int c = 0; c < nch; ++c) {
+        for (int c = hf ? (nch + 1) >> 1 : 0; c < c1; ++c) {
           uint32_t x[32];
           tmem_ld_32cols(tbase + static_cast<uint32_t>(32 * c), x);
           tmem_ld_wait();
-          const int v0 = vbase + 32 * c;
-          // vocabulary rows past the group's (stale stage bytes) or past V
-          const int nvalid = min(min(32, gr - 32 * c), p.V - v0);
-          float cm = kNegBig;
-          int ci = 0;
-#pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            const float z = __uint_as_float(x[k]) * rs;
-            if (k < nvalid && z > cm) {
-              cm = z;
-              ci = k;
-            }
-          }
-          if (cm > m) {  // strictly: an equal maximum keeps the lower index
-            s *= fast_exp2(m - cm);
-            m = cm;
-            ix = v0 + ci;
-          }
-          float cs = 0.0f;
-#pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            const float z = __uint_as_float(x[k]) * rs;
-            cs += k < nvalid ? fast_exp2(z - m) : 0.0f;
-          }
-          s += cs;
+          fold_row32(m, s, ix, x, rs, vbase + 32 * c, nrow - 32 * c);
         }
       }
       tc_fence_before();
@@ -445,7 +429,17 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
       if (lane == 0) mbar_arrive(&sm.acce[racc.slot]);
       racc.next(2);
     }
-    if (ok && row < M) {
+    // The second half's triples go through shared memory to the first's.
+    __shared__ float s_x[3][kRowsM];
+    if (ok && hf) {
+      s_x[0][row] = m;
+      s_x[1][row] = s;
+      s_x[2][row] = __int_as_float(ix);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sm.xch);
+    } else if (ok && active &&
+               mbar_wait(sm.xch, 0, sm.abort, p.err, kErrWaitEpi) && row < M) {
+      merge_tri(m, s, ix, s_x[0][row], s_x[1][row], __float_as_int(s_x[2][row]));
       // The previous step's commit reads the same partial buffer.
       grid_dependency_wait();
       p.part[static_cast<size_t>(row) * gridDim.x + cta] = make_float4(m, s, __int_as_float(ix), 0.0f);

@@ -28,15 +28,16 @@ __device__ __forceinline__ float sumsq8(uint4 x) {
 }
 
 // Final RMSNorm row scales 1 / sqrt(mean h^2 + eps) of rows [0, M) of the
-// [M, H] bf16 rows `hid` into s_scale (shared memory), by the four epilogue
-// warps of an LM-head kernel (ew = 0..3, each a whole warp; every one must
+// [M, H] bf16 rows `hid` into s_scale (shared memory), by the kWarps epilogue
+// warps of an LM-head kernel (ew = 0.., each a whole warp; every one must
 // call it), which then meet at named barrier 1: a row at a time per warp, 32
 // lanes with eight 16-byte loads each in flight.
+template <int kWarps>
 __device__ __forceinline__ void epilogue_row_scales(const __nv_bfloat16* hid, int M, int H,
                                                     float eps, float* s_scale, int ew,
                                                     int lane) {
   const int nvec = H / 8;
-  for (int r = ew; r < M; r += 4) {
+  for (int r = ew; r < M; r += kWarps) {
     const uint4* src = reinterpret_cast<const uint4*>(hid + static_cast<size_t>(r) * H);
     float ss = 0.0f;
     for (int v0 = lane; v0 < nvec; v0 += 32 * 8) {
@@ -53,7 +54,7 @@ __device__ __forceinline__ void epilogue_row_scales(const __nv_bfloat16* hid, in
     for (int off = 16; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
     if (lane == 0) s_scale[r] = rsqrtf(ss / static_cast<float>(H) + eps);
   }
-  asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarps) : "memory");  // the epilogue warps
 }
 
 __device__ __forceinline__ float fast_exp2(float x) {

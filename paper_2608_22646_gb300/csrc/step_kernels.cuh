@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kShardThreads) shard_merge_kernel(const ShardM
 
 // ------------------------------------------------------ merge + commit (K3) --
 
-// One CTA per sequence: merge_commit_sequence for sequence blockIdx.x, then the
+// One CTA per sequence: merge_commit for sequence blockIdx.x, then the
 // last CTA to finish (atomic ticket; none needed for a single CTA) builds the
 // next step's list and publishes the step.
 __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const CommitParams p) {
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const Comm
   int M = 0;
   if (p.prefetch_state) {
     M = p.t == 0 ? p.B * p.P : __ldcg(p.d_M);
-    commit_load(p, blockIdx.x, cs);
+    commit_load(p, blockIdx.x, 1, cs);
   }
   // With prefetch_state the CTA is resident long before the partials are
   // there: it makes a first pass over whatever the buffers hold, writing
@@ -375,7 +375,10 @@ __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const Comm
   for (int pass = p.prefetch_state ? 0 : 1; pass < 2; ++pass) {
     const bool real = pass == 1;
     if (real) grid_dependency_wait();  // partials of this step (and state of the previous one)
-    if (!p.prefetch_state) M = *p.d_M;
+    if (!p.prefetch_state) {
+      M = *p.d_M;
+      commit_load(p, blockIdx.x, 1, cs);
+    }
     const float4* part = p.part;
     int n_part = p.n_part;
     if (M >= p.pair_min_M) {
@@ -385,8 +388,7 @@ __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const Comm
         n_part = 1;
       }
     }
-    merge_commit_sequence<kCommitPPW>(p, blockIdx.x, cs, part, n_part, nullptr,
-                                      p.prefetch_state != 0, real);
+    merge_commit<kCommitPPW>(p, blockIdx.x, 1, cs, part, n_part, real);
     if (gridDim.x > 1 && real) {
       if (threadIdx.x == 0) {
         __threadfence();
