@@ -33,8 +33,8 @@
  * merge + commit.  The LM head is the CTA-pair
  * kernel (tcgen05 cta_group::2), which picks its orientation per step from
  * the masked-row count M: the rows as MMA N in row tiles of equal width (a
- * multiple of 32) while that width is at most 192, else as MMA M in 256-row
- * tiles.  A kernel that merges each row's per-tile partials follows it only
+ * multiple of 32) while that width is at most a limit that grows with H (224
+ * from H = 3072 on), else as MMA M in 256-row tiles.  A kernel that merges each row's per-tile partials follows it only
  * in contexts where some step size leaves more than one partial per pair and
  * CTA to merge.  CAI_PAIR_SWAP=0 keeps the pair kernel unswapped and moves
  * the steps below 32 rows to the single-CTA swapped-operand kernel (launched
@@ -197,7 +197,10 @@ typedef struct cai_stats {
   int32_t pair_grid;        /* CTAs of the CTA-pair LM head (0: not used)          */
   int32_t pair_swap_max_n;  /* steps whose tile width in the swapped orientation
                                (masked rows in the MMA N dimension) is at most
-                               this run swapped on the pair LM head (0: never)     */
+                               this may run swapped on the pair LM head (0: never);
+                               unless CAI_PAIR_SWAP_MAX_N is set, the limit in use
+                               follows H: 0 below 384, 64 below 768, 96 below 1536,
+                               192 below 3072, then 224                            */
   int32_t pair_stages;      /* pipeline stages of the pair LM head                 */
   int32_t head_rows;        /* 1: single-kernel steps run the LM head with the rows
                                as the MMA's A operand (B P <= 128), 0: otherwise   */

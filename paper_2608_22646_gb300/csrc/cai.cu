@@ -808,6 +808,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   if (shard && c->swap_max_n < kSwapColStep) c->swap_max_n = 192;
   c->stats.pair_swap_max_n = c->swap_max_n;
   c->swap_on = c->swap_max_n > 0;
+  if (c->swap_on && pair_swap_env() == 0) c->swap_max_n = pair_swap_width(cfg->H);
   c->pair_kernel = c->norm ? lm_head_pair_kernel<true> : lm_head_pair_kernel<false>;
 
   // LM-head launch shape.  N chunk (positions per MMA), grid (one CTA per SM,

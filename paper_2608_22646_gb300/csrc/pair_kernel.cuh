@@ -152,6 +152,18 @@ __host__ __device__ inline bool pair_swapped(int M, int swap_max_n) {
   return M > 0 && swap_tile_cols(M, pair_row_tiles(M)) <= swap_max_n;
 }
 
+// Widest swapped tile by default, from the length of the contraction: the
+// swapped orientation pads fewer rows, but its epilogue takes longer per tile,
+// and the shorter K is the less of it is hidden.  0: always unswapped.
+// Measured, microseconds a step, swapped against unswapped: H = 256 (V = 4096)
+// N = 32 13.7 / 12.6; H = 512 (22000) N = 64 17.4 / 17.5, N = 96 18.5 / 17.6;
+// H = 1024 (50003) N = 96 27.2 / 28.5, N = 160 29.9 / 28.8; H = 2048 (50003)
+// N = 192 48.3 / 46.3, two tiles of 160 57.5 / 66.5; H = 4096 (126464) N = 224
+// 171 / 172, two tiles of 224 271 / 299, N = 256 183 / 182.
+__host__ __device__ inline int pair_swap_width(int H) {
+  return H < 384 ? 0 : H < 768 ? 64 : H < 1536 ? 96 : H < 3072 ? 192 : 224;
+}
+
 // Partials per row written by a pair step with M rows on n_pairs pairs: one
 // per pair of the row's tile (two in the swapped orientation, one per CTA)
 // when n_pairs is a multiple of the row-tile count, else 0 (one per

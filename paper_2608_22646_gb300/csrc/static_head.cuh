@@ -28,7 +28,6 @@ namespace {
 constexpr int kStaticMaxRows = 256;   // rows per call (one row tile)
 constexpr int kStaticMaxParts = 160;  // partials per row: one per CTA
 constexpr int kStaticStages = 6;      // ring slots of kPairStageBytes
-constexpr int kStaticSwapMaxN = 192;  // widest swapped tile, as the contexts' default
 constexpr int kStaticMaxDevices = 64;
 
 // The whole scratch of the entry point: partial triples [row][CTA], plus one
@@ -199,13 +198,13 @@ extern "C" int cai_head_rows_static(const void* W, int32_t V, int32_t H, const v
   pp.H = H;
   pp.n_vt = pp.n_vt1;
   pp.min_M = 1;
-  pp.swap_max_n = kStaticSwapMaxN;
-  pp.n_stages = d->stages;
+  pp.swap_max_n = pair_swap_width(H);
+  pp.n_stages = d->stages;  // the ring of smem sized with the exchange buffer
   pp.ring_max = 8;
   pp.M_fixed = M;
   pp.w_dx = kPairBlockK;
   pp.w_ry = 1;
-  const bool swap = pair_swapped(M, kStaticSwapMaxN);
+  const bool swap = pair_swapped(M, pp.swap_max_n);
   const int rows_box = swap ? swap_tile_cols(M, 1) / 2 : kPairHalf;
   CUtensorMap tm_w, tm_r;
   if (!encode(&tm_w, W, static_cast<uint64_t>(V), static_cast<uint64_t>(H), pp.th1) ||
