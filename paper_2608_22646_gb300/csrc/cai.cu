@@ -419,7 +419,9 @@ float theta_token_of(const cai_config& c, double theta_block, int p) {
 CommitParams commit_params(cai_ctx* c, int t, int64_t step_id) {
   const cai_config& cfg = c->cfg;
   CommitParams cp{};
-  cp.part = c->part;
+  // Single-kernel steps alternate between two partial buffers and tickets.
+  const int alt = c->fused ? static_cast<int>(step_id & 1) : 0;
+  cp.part = c->part + static_cast<size_t>(alt) * c->rows_cap * c->G;
   cp.n_part = c->G;
   cp.rowres = c->rowres;
   cp.pair_pairs = c->pair_grid / 2;
@@ -435,7 +437,7 @@ CommitParams commit_params(cai_ctx* c, int t, int64_t step_id) {
   cp.row_of = c->row_of;
   cp.d_M = c->d_M;
   cp.m_hist_slot = c->st.m_hist + c->blk * cfg.T + t;
-  cp.ticket = c->ticket;
+  cp.ticket = c->ticket + alt;
   cp.pub = c->pub;
   cp.hf = c->hf_dev;
   cp.err = c->err;
@@ -662,7 +664,7 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
   }
   hp.prefetch = c->use_pair ? 0 : 1;
   hp.first = first ? 1 : 0;
-  hp.part = c->part;
+  hp.part = c->part;  // (single-kernel step: cp.part, below)
   hp.err = c->err;
   hp.V = cfg.V;
   hp.H = cfg.H;
@@ -677,7 +679,10 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
   hp.hid = static_cast<const __nv_bfloat16*>(hid);
   hp.norm_eps = c->norm_eps;
   const CommitParams cp = commit_params(c, t, step_id);
-  if (c->fused) hp.cp = cp;
+  if (c->fused) {
+    hp.cp = cp;
+    hp.part = const_cast<float4*>(cp.part);
+  }
   if (c->profiling) cudaEventRecord(ev[1], stream);
   if (c->head_in_step) {
     const CUtensorMap& tm_rows =
@@ -1005,7 +1010,12 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   CAI_ALLOC(c->list, int, c->BP)
   CAI_ALLOC(c->row_of, int, c->BP)
   CAI_ALLOC(c->d_M, int, 1)
-  CAI_ALLOC(c->ticket, unsigned, 1)
+  CAI_ALLOC(c->ticket, unsigned, 2)
+  if (cudaMemset(c->ticket, 0, 8) != cudaSuccess) {  // every step leaves it at zero
+    release(c);
+    delete c;
+    return CAI_ERR_CUDA;
+  }
   CAI_ALLOC(c->pub, unsigned long long, 1)
   CAI_ALLOC(c->err, uint32_t, 1)
   CAI_ALLOC(c->hc, __nv_bfloat16, static_cast<size_t>(c->rows_cap) * cfg->H)
@@ -1017,6 +1027,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     part_cols = k * c->n_vt > part_cols ? k * c->n_vt : part_cols;
     part_cols = k * (c->pair_grid / 2) > part_cols ? k * (c->pair_grid / 2) : part_cols;
   }
+  if (c->fused) part_cols *= 2;  // two buffers, alternating by step
   CAI_ALLOC(c->part, float4, static_cast<size_t>(c->rows_cap) * part_cols)
   if (c->use_pair) {
     CAI_ALLOC(c->wt, uint8_t,
@@ -1238,7 +1249,6 @@ int cai_reset(cai_ctx* c, void* stream_v) {
   fill(c->st.run, BL, 0u);
   fill(c->st.stable, BL * 2, ~0u);
   fill(c->st.drift, BN * cfg.T * 4, ~0u);  // NaN
-  fill(c->ticket, 4, 0u);
   fill(c->pub, 8, 0u);
   fill(c->err, 4, 0u);
   fill(c->d_M, 4, 0u);

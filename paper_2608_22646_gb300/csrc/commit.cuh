@@ -75,7 +75,7 @@ struct CommitParams {
   int* row_of;
   int* d_M;
   int* m_hist_slot;       // this step's M_t (written by the single-kernel step)
-  unsigned* ticket;       // zero between launches
+  unsigned* ticket;       // zero between steps that use it (atomicInc wraps it)
   unsigned long long* pub;  // (step id + 1) << 32 | masked rows left, written by finish_step
   HostFlag* hf;           // device alias of the mapped host record
   uint32_t* err;
@@ -101,8 +101,9 @@ __device__ __forceinline__ int budget_tier(float s, int p, int half, int late) {
 // sequences, at most kMaxP of them, sequence by sequence.
 struct CommitSmem {
   int tok[kMaxP];      // token after this step (kMask while masked)
-  int cand[kMaxP];     // argmax of the previous decoded step, then of this step
-  float conf[kMaxP];   // confidence of this step
+  int cand[kMaxP];     // diagnostics: argmax of the previous decoded step
+  float conf[kMaxP];   // confidence and argmax of this step (merge_rows)
+  int idx[kMaxP];
   int row[kMaxP];      // partial row of the position in this step (masked positions)
   uint8_t bud[kMaxP];  // budget before this step
   uint8_t run[kMaxP];  // diagnostics: same-argmax run before this step
@@ -147,27 +148,56 @@ __device__ __forceinline__ void commit_load(const CommitParams& p, int b0, int n
   }
 }
 
-// One step of Algorithm 1 for the sequences [b0, b0 + nb) that commit_load has
-// read into cs (nb P <= kMaxP), by the whole calling CTA (blockDim.x a multiple
-// of 32; every thread must call it).  Warps merge the partials of the
-// still-masked positions (kPPW at a time, all loads issued before any merge)
-// and lane 0 applies the commit rule (Box 6, Eq. position_commit, with the
-// step-zero init of Boxes 2 and 5); one thread per sequence updates the
-// low-yield counter and the exit state (Box 7, Algorithm 1).  Global state is
-// only written, never re-read.  Leaves in cs, for every thread, the positions
-// decoded and those still masked afterwards in running sequences.  With `real`
-// false nothing outside the CTA is written and cs keeps its contents: a pass
-// over stale partials that brings the code into the instruction caches.
-template <int kPPW = kPosPerWarp>
-__device__ void merge_commit(const CommitParams& p, int b0, int nb, CommitSmem& cs,
-                             const float4* part, int n_part, bool real = true) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// The commit rule (Box 6, Eq. position_commit, with the step-zero init of Boxes
+// 2 and 5) for position i of cs with confidence c and argmax ix, by one thread.
+__device__ __forceinline__ void commit_position(const CommitParams& p, int b0, CommitSmem& cs,
+                                                int i, float c, int ix) {
+  const int sq = i / p.P, pp = i - sq * p.P;
+  const size_t g = static_cast<size_t>(b0 + sq) * p.L + p.blk * p.P + pp;
+  int bud = cs.bud[i];
+  if (p.t == 0) {
+    bud = budget_tier(c, pp, p.budget_half, p.budget_late);
+    p.st.s0[g] = c;
+    p.st.budget[g] = static_cast<uint8_t>(bud);
+  }
+  if ((p.flags & kFlagDiag) != 0) {
+    // Section 2.1: stable once the argmax has held for three decoded steps.
+    const int run = (p.t > 0 && cs.cand[i] == ix) ? cs.run[i] + 1 : 1;
+    p.st.run[g] = static_cast<uint8_t>(run < 255 ? run : 255);
+    if (run >= 3 && cs.stable[i] < 0) p.st.stable[g] = static_cast<int16_t>(p.t);
+  }
+  p.st.conf[g] = c;
+  p.st.cand[g] = ix;
+  cs.conf[i] = c;
+  cs.idx[i] = ix;
+  const bool by_conf = c >= p.theta_tab[pp];
+  const bool by_budget = (p.flags & kFlagGating) != 0 && p.t >= bud;
+  if (by_conf || by_budget) {
+    cs.tok[i] = ix;
+    p.st.tok[g] = ix;
+    p.st.cstep[g] = static_cast<int16_t>(p.t);
+    atomicAdd(&cs.eta[sq], 1);
+  } else {
+    atomicAdd(&cs.left[sq], 1);
+  }
+}
+
+// Merges the partials of the block's positions of sequences [b0, b0 + nb) (nb P
+// <= kMaxP), by the whole calling CTA (blockDim.x a multiple of 32): a warp per
+// position, kPPW at a time, all loads issued before any merge.  kAll: every
+// position, in the order of the block (rows of a single-kernel step), into
+// cs.conf and cs.idx, which needs no state.  Else the still-masked positions of
+// running sequences, at the rows commit_load has read, each committed by its
+// warp's first lane as soon as it is merged (a second pass with a thread per
+// position cost 0.8 to 1.2 us a step).  With `real` false nothing outside the
+// CTA is written and cs is left alone: a pass over stale partials that brings
+// the code into the instruction caches.
+template <int kPPW, bool kAll>
+__device__ void merge_rows(const CommitParams& p, int b0, int nb, CommitSmem& cs,
+                           const float4* part, int n_part, bool real = true) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
   const int n = nb * p.P;
-  const bool diag = (p.flags & kFlagDiag) != 0;
-  const bool gating = (p.flags & kFlagGating) != 0;
-  __syncthreads();
-
   for (int base = warp; base < n; base += nwarps * kPPW) {
     int row[kPPW];
     float4 q[kPPW][kPartPerLane];
@@ -175,7 +205,9 @@ __device__ void merge_commit(const CommitParams& p, int b0, int nb, CommitSmem& 
     for (int j = 0; j < kPPW; ++j) {
       const int i = base + j * nwarps;
       row[j] = -1;
-      if (i < n && cs.tok[i] == kMask && cs.running[i / p.P]) {
+      if (kAll) {
+        if (i < n) row[j] = b0 * p.P + i;
+      } else if (i < n && cs.tok[i] == kMask && cs.running[i / p.P]) {
         row[j] = cs.row[i];
         if (!CAI_IN_RANGE(row[j] < p.B * p.P, p.err)) row[j] = -2;
         if (row[j] < 0) {
@@ -198,7 +230,6 @@ __device__ void merge_commit(const CommitParams& p, int b0, int nb, CommitSmem& 
 #pragma unroll
     for (int j = 0; j < kPPW; ++j) {
       if (row[j] < 0) continue;  // warp-uniform
-      const int i = base + j * nwarps;
       for (int k = lane + 32 * kPartPerLane; k < n_part; k += 32) {
         const float4 r = __ldcg(part + static_cast<size_t>(row[j]) * n_part + k);
         int i0 = __float_as_int(q[j][0].z);
@@ -209,39 +240,31 @@ __device__ void merge_commit(const CommitParams& p, int b0, int nb, CommitSmem& 
       float m, s;
       int ix;
       warp_merge(q[j], m, s, ix);
-      if (lane == 0 && real) {
-        const int sq = i / p.P, pp = i - sq * p.P;
-        const size_t g = static_cast<size_t>(b0 + sq) * p.L + p.blk * p.P + pp;
-        const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)
-        int bud = cs.bud[i];
-        if (p.t == 0) {
-          bud = budget_tier(c, pp, p.budget_half, p.budget_late);
-          p.st.s0[g] = c;
-          p.st.budget[g] = static_cast<uint8_t>(bud);
-        }
-        if (diag) {
-          // Section 2.1: stable once the argmax has held for three decoded steps.
-          const int run = (p.t > 0 && cs.cand[i] == ix) ? cs.run[i] + 1 : 1;
-          p.st.run[g] = static_cast<uint8_t>(run < 255 ? run : 255);
-          if (run >= 3 && cs.stable[i] < 0) p.st.stable[g] = static_cast<int16_t>(p.t);
-        }
-        p.st.conf[g] = c;
-        p.st.cand[g] = ix;
-        cs.conf[i] = c;
-        cs.cand[i] = ix;
-        const bool by_conf = c >= p.theta_tab[pp];
-        const bool by_budget = gating && p.t >= bud;
-        if (by_conf || by_budget) {
-          cs.tok[i] = ix;
-          p.st.tok[g] = ix;
-          p.st.cstep[g] = static_cast<int16_t>(p.t);
-          atomicAdd(&cs.eta[sq], 1);
-        } else {
-          atomicAdd(&cs.left[sq], 1);
+      const int i = base + j * nwarps;
+      const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)
+      if (lane == 0) {
+        if (kAll) {
+          cs.conf[i] = c;
+          cs.idx[i] = ix;
+        } else if (real) {
+          commit_position(p, b0, cs, i, c, ix);
         }
       }
     }
   }
+}
+
+// The end of a step of Algorithm 1 for the sequences [b0, b0 + nb) once their
+// positions are committed (commit_position), by the whole calling CTA; every
+// thread must call it.  One thread per sequence updates the low-yield counter
+// and the exit state (Box 7, Algorithm 1).  Global state is only written, never
+// re-read.  Leaves in cs, for every thread, the positions decoded and those
+// still masked afterwards in running sequences.  `real` as in merge_rows.
+__device__ void finish_sequences(const CommitParams& p, int b0, int nb, CommitSmem& cs,
+                                 bool real = true) {
+  const int tid = threadIdx.x;
+  const int n = nb * p.P;
+  const bool gating = (p.flags & kFlagGating) != 0;
   __syncthreads();
   if (!real) return;
   bool exits = false;
@@ -277,7 +300,7 @@ __device__ void merge_commit(const CommitParams& p, int b0, int nb, CommitSmem& 
     if (reason == kRunning || cs.tok[i] != kMask) continue;
     const size_t g = static_cast<size_t>(b0 + sq) * p.L + p.blk * p.P + (i - sq * p.P);
     if ((reason == kExitGrind && cs.conf[i] > p.theta_fb) || (p.flags & kFlagFlush)) {
-      p.st.tok[g] = cs.cand[i];
+      p.st.tok[g] = cs.idx[i];
       p.st.cstep[g] = static_cast<int16_t>(p.t);
     } else {
       atomicAdd(&cs.unres[sq], 1);
@@ -341,16 +364,15 @@ __device__ int build_masked_list(const int* tok, const int* exit_reason, int* li
 
 // End of a step, by the last CTA: the next step's list (multi-kernel step
 // only; the single-kernel step decodes every row and needs none), M_{t+1},
-// the reset ticket and the host-visible record.  `remaining` is the masked
+// and the host-visible record.  `remaining` is the masked
 // count of running sequences when the caller already knows it (-1: count).
-// `real` as in merge_commit.
+// `real` as in merge_rows.
 __device__ void finish_step(const CommitParams& p, int remaining = -1, bool real = true) {
   const int n = remaining >= 0 ? remaining
                                : build_masked_list(p.st.tok, p.st.exit_reason, p.list, p.row_of,
                                                    p.B, p.P, p.L, p.n_blocks, p.blk, real);
   if (threadIdx.x == 0 && real) {
     *p.d_M = n;
-    *p.ticket = 0u;
     const bool err = *reinterpret_cast<volatile uint32_t*>(p.err) != 0u;
     // The host uses this word only for control flow; it reads the state
     // itself through stream-ordered copies, so no system fence is needed.

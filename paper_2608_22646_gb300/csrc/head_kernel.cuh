@@ -288,24 +288,48 @@ struct Ring {
   }
 };
 
+// Single-kernel steps alternate between two partial buffers and tickets
+// (step id & 1), so that a step's CTAs finish without waiting for the previous
+// step's commit; only the CTA that commits waits for it.  Those a step uses
+// were last used two steps before: free once that step's commit has published
+// its word (load_pub), or when the previous kernel has completed.  Step zero of
+// a block waits in any case (a reset may still be under way).
+__device__ __forceinline__ bool step_buffers_free(const CommitParams& cp, bool first) {
+  const uint32_t id = static_cast<uint32_t>(load_pub(cp.pub) >> 32);
+  return !first && static_cast<int32_t>(id - static_cast<uint32_t>(cp.step_id - 1)) >= 0;
+}
+
 // Single-kernel step, end of every CTA: the last CTA to finish (atomic
-// ticket, no waiting) merges the partials and commits the step for every
-// sequence, after the previous step's commit (state, ticket) is complete.
+// ticket, no waiting) merges every row's partials, then, after the previous
+// step's commit (the state) is complete, commits the step for every sequence.
 // `free_smem` is at least sizeof(CommitSmem) bytes of shared memory that no
-// copy or MMA touches any more (the drained W ring).
-__device__ __forceinline__ void fused_step_commit(const CommitParams& cp, uint8_t* free_smem) {
-  grid_dependency_wait();
+// copy or MMA touches any more (the drained W ring); `free_now`, of thread 0:
+// step_buffers_free held.
+//
+// What bounds small models back to back is this chain from one step's commit
+// to the next: with one buffer, waits before the partials and the ticket, and
+// state, partials and rule one after the other, a step of 256 x 4096 with 16
+// rows took 8.8 us.
+__device__ __forceinline__ void fused_step_commit(const CommitParams& cp, uint8_t* free_smem,
+                                                  bool free_now) {
   __shared__ int s_last;
   if (threadIdx.x == 0) {
+    if (!free_now) grid_dependency_wait();
     __threadfence();
-    s_last = atomicAdd(cp.ticket, 1u) == gridDim.x - 1;
+    s_last = atomicInc(cp.ticket, gridDim.x - 1) == gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   CommitSmem& cs = *reinterpret_cast<CommitSmem*>(free_smem);
+  merge_rows<kPosPerWarp, true>(cp, 0, cp.B, cs, cp.part, cp.n_part);
+  grid_dependency_wait();
   commit_load(cp, 0, cp.B, cs);
-  merge_commit(cp, 0, cp.B, cs, cp.part, cp.n_part);
+  __syncthreads();
+  for (int i = threadIdx.x; i < cp.B * cp.P; i += blockDim.x)  // a thread per position
+    if (cs.tok[i] == kMask && cs.running[i / cp.P])
+      commit_position(cp, 0, cs, i, cs.conf[i], cs.idx[i]);
+  finish_sequences(cp, 0, cp.B, cs);
   if (threadIdx.x == 0) *cp.m_hist_slot = cs.decoded;
   finish_step(cp, cs.remaining);
 }
@@ -723,7 +747,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
     tmem_dealloc(tmem_base, static_cast<uint32_t>(p.tmem_cols));
   }
 
-  if (p.fused) fused_step_commit(p.cp, sm.a);
+  if (p.fused) fused_step_commit(p.cp, sm.a, threadIdx.x == 0 && step_buffers_free(p.cp, p.first != 0));
 }
 
 }  // namespace cai

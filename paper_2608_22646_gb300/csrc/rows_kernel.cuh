@@ -245,6 +245,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *sm.tmem_slot;
 
+  bool buffers_free = false;  // thread 0: see fused_step_commit
   if (warp == 0) {
     // -------------------------------------------------------- producer --
     // The whole warp runs the loop and one lane issues (see the pair
@@ -325,6 +326,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
       }
     }
     __syncwarp();
+    if (lane == 0) buffers_free = step_buffers_free(p.cp, p.first != 0);
   } else if (warp == 1) {
     // ------------------------------------------------------ MMA issuer --
     const bool leader = elect_one();
@@ -397,7 +399,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     }
     Ring racc;
     bool ok = true;
+    bool free_now = false;  // looked up early: the load is not waited for at the end
     for (int g = 0; g < pl.n_groups; ++g) {
+      if (g == pl.n_groups - 1) free_now = step_buffers_free(p.cp, p.first != 0);
       if (!mbar_wait(&sm.accf[racc.slot], racc.phase, sm.abort, p.err, kErrWaitAccFull)) {
         ok = false;
         break;
@@ -440,8 +444,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     } else if (ok && active &&
                mbar_wait(sm.xch, 0, sm.abort, p.err, kErrWaitEpi) && row < M) {
       merge_tri(m, s, ix, s_x[0][row], s_x[1][row], __float_as_int(s_x[2][row]));
-      // The previous step's commit reads the same partial buffer.
-      grid_dependency_wait();
+      // The step before last read the same partial buffer.
+      if (!free_now && !step_buffers_free(p.cp, p.first != 0)) grid_dependency_wait();
       p.part[static_cast<size_t>(row) * gridDim.x + cta] = make_float4(m, s, __int_as_float(ix), 0.0f);
     }
   }
@@ -452,7 +456,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     tc_fence_after();
     tmem_dealloc(tmem_base, kRowsTmemCols);
   }
-  fused_step_commit(p.cp, sm.w);
+  fused_step_commit(p.cp, sm.w, buffers_free);
 }
 
 }  // namespace cai

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(32 * kDriftRowsPerCta) drift_kernel(const Drif
 // each rounded up to 16 bytes (every buffer is padded to 256).  One launch
 // instead of a memset per array, whose 19 launches of ~1.5 us each a toy-sized
 // generation spent a tenth of its time on.
-constexpr int kResetFills = 19;
+constexpr int kResetFills = 18;
 constexpr int kResetThreads = 256;
 struct ResetParams {
   uint4* ptr[kResetFills];
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kShardThreads) shard_merge_kernel(const ShardM
 
 // ------------------------------------------------------ merge + commit (K3) --
 
-// One CTA per sequence: merge_commit for sequence blockIdx.x, then the
+// One CTA per sequence: merge and commit of sequence blockIdx.x, then the
 // last CTA to finish (atomic ticket; none needed for a single CTA) builds the
 // next step's list and publishes the step.
 __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const CommitParams p) {
@@ -388,11 +388,13 @@ __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const Comm
         n_part = 1;
       }
     }
-    merge_commit<kCommitPPW>(p, blockIdx.x, 1, cs, part, n_part, real);
+    __syncthreads();  // cs
+    merge_rows<kCommitPPW, false>(p, blockIdx.x, 1, cs, part, n_part, real);
+    finish_sequences(p, blockIdx.x, 1, cs, real);
     if (gridDim.x > 1 && real) {
       if (threadIdx.x == 0) {
         __threadfence();
-        s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+        s_last = atomicInc(p.ticket, gridDim.x - 1) == gridDim.x - 1;
       }
       __syncthreads();
       if (!s_last) return;
