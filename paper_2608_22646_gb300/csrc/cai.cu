@@ -36,12 +36,12 @@ std::atomic<int> g_head_grid_limit{0};
 // the rows to 128 anyway, and the next step's weight stream runs under the
 // commit.  Measured, microseconds a step back to back, single- against
 // multi-kernel with every row masked (multi-kernel at 8 rows in brackets):
-// 96 rows, 4096 x 126464 135 against 159 (152), 1024 x 50003 18.5 against 28.2
-// (21); 128 rows, 144 against 161, 3584 x 152064 145 against 165, 1024 x 22000
-// 18.2 against 21.6 (15); alone 165.8 against 174 at 96 rows and 174.6 against
-// 174.6 at 128.  With a weight of a few MB both are chains of latencies, and
-// above 64 rows the multi-kernel one gets shorter as rows commit (256 x 4096,
-// 128 rows: 15.1 against 15.7, 13.8 at 8 rows).
+// 96 rows, 4096 x 126464 134 against 159 (152), 1024 x 50003 18.4 against 28.2
+// (21); 128 rows, 142 against 161, 3584 x 152064 145 against 165, 1024 x 22000
+// 11.7 against 21.6 (15); alone 165.8 against 174 at 96 rows and 174.6 against
+// 174.6 at 128.  With a weight of a few MB both are short chains of latencies
+// that differ little, and above 64 rows the multi-kernel step stays: it gets
+// shorter as rows commit.
 constexpr int kFusedMaxRows = 64;       // any weight
 constexpr int kFusedMaxRowsLarge = 128; // weights of at least ...
 constexpr long long kFusedLargeBytes = 8ll << 20;
@@ -1097,20 +1097,22 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     w_src = w_tmp;
   }
   {
-    const long long n_chunks = static_cast<long long>(units) * kUnitRows * cfg->H / 8;
+    const int pack_grid = 8 * sms;
     if (c->rows_head)
-      pack_weight_rows_kernel<<<4 * sms, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      pack_weight_rows_kernel<<<pack_grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wpk), cfg->V, cfg->H, units,
-          c->G, n_chunks, g_dev);
+          c->G, g_dev);
     else if (c->head_in_step)
-      pack_weight_kernel<<<4 * sms, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      pack_weight_kernel<<<pack_grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wpk), cfg->V, cfg->H, units,
-          c->G, c->gmax, n_chunks, g_dev);
+          c->G, c->gmax, g_dev);
     if (c->use_pair)
-      pack_w_tiles_kernel<<<4 * sms, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      pack_w_tiles_kernel<<<pack_grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wt), cfg->V, cfg->H,
           pair_w_run(cfg->V, c->pair_th1),
-          pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1)) * (kPairBlockK / 8), g_dev);
+          static_cast<int>(pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1)) /
+                           (cfg->H / kPairBlockK) / kUnitRows),
+          g_dev);
     const cudaError_t e1 = cudaGetLastError();
     const cudaError_t e2 = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
     if (w_tmp) cudaFree(w_tmp);

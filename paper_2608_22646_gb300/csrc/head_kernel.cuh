@@ -180,42 +180,70 @@ __device__ __forceinline__ uint4 scale_chunk(uint4 w, const __nv_bfloat16* g) {
   return w;
 }
 
-// Pack W [V, H] (row-major bf16) for a grid of G CTAs over `units` units of
-// kUnitRows rows and groups of up to gmax tiles.  Inside a stage block, row r's
-// 16-byte chunk c (k = 8c..8c+7 of the block's 64) sits at
-// r * 128 + ((c ^ (r & 7)) * 16): the 128-byte swizzle of 8-row, 1024-byte
-// atoms.  Rows >= V are zero.  One thread per destination 16-byte chunk;
-// n_chunks = units * kUnitRows * H / 8.
-__global__ void pack_weight_kernel(const uint4* __restrict__ W, uint4* __restrict__ out, int V,
-                                   int H, int units, int G, int gmax, long long n_chunks,
-                                   const __nv_bfloat16* __restrict__ gw) {
-  const long long unit_bytes = 2ll * kUnitRows * H;
-  for (long long d = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; d < n_chunks;
-       d += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long byte = d * 16;
-    const int u = static_cast<int>(byte / unit_bytes);
-    // CTA owning unit u: the largest c with unit_begin(c) <= u.
-    int c = static_cast<int>((static_cast<long long>(u) * G) / units);
-    while (c + 1 < G && unit_begin(c + 1, units, G) <= u) ++c;
-    while (c > 0 && unit_begin(c, units, G) > u) --c;
-    const CtaPlan pl = cta_plan(c, units, G, gmax);
-    const long long off = byte - static_cast<long long>(pl.u0) * unit_bytes;
-    const long long group_bytes = static_cast<long long>(pl.gsz) * kRowsPerTile * 2 * H;
-    const int g = static_cast<int>(off / group_bytes);
-    const long long rem = off - static_cast<long long>(g) * group_bytes;
-    const int grow = pl.group_rows(g);
-    const int kb = static_cast<int>(rem / (grow * 128));
-    const int rem2 = static_cast<int>(rem - static_cast<long long>(kb) * grow * 128);
-    const int t = pl.group_first(g) + rem2 / kATileBytes;
-    const int inblk = rem2 % kATileBytes;
-    const int r = inblk >> 7;
-    const int cl = ((inblk >> 4) & 7) ^ (r & 7);
-    const long long v = static_cast<long long>(pl.row0()) + t * kRowsPerTile + r;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    if (v < V) val = W[(v * H + static_cast<long long>(kb) * kBlockK) / 8 + cl];
-    if (gw) val = scale_chunk(val, gw + kb * kBlockK + cl * 8);
-    out[d] = val;
+// Packing of W [V, H] (row-major bf16) into the layouts of the LM-head kernels,
+// once per context.  All of them keep the kUnitRows rows of a unit together: K
+// block kb of a unit is one 1 KiB atom at base + kb stride, in the 128-byte
+// swizzle (16-byte chunk c of row r at r * 128 + (c ^ (r & 7)) * 16); only the
+// base and the stride differ.
+struct PackDst {
+  long long base, stride;  // bytes
+};
+
+// One CTA packs one unit at a time: the place of the unit is worked out once,
+// and a thread moves the 16-byte chunks i, i + blockDim.x, ... of the unit's H
+// columns, eight loads in flight.  Rows >= V are zero; gw (bf16 [H], or null)
+// is the final-norm weight folded in.  Bound by memory.  With the place worked
+// out per chunk (several 64-bit divisions each) cai_init of 126464 x 4096 took
+// 1.75 ms for the rows-operand layout and 1.04 ms for the pair kernel's; both
+// now take 0.9 ms.
+template <typename Place>
+__device__ __forceinline__ void pack_units(const uint4* __restrict__ W, uint4* __restrict__ out,
+                                           int V, int H, int units,
+                                           const __nv_bfloat16* __restrict__ gw, Place place) {
+  constexpr int kVecs = 8;
+  const int n = H / kBlockK * 64;  // chunks of a unit
+  for (int u = blockIdx.x; u < units; u += gridDim.x) {
+    const PackDst d = place(u);
+    for (int i0 = threadIdx.x; i0 < n; i0 += kVecs * blockDim.x) {
+      uint4 x[kVecs];
+#pragma unroll
+      for (int j = 0; j < kVecs; ++j) {
+        const int i = i0 + j * blockDim.x;
+        const int kb = i >> 6, r = (i >> 3) & 7, c = (i & 7) ^ r;
+        const long long v = static_cast<long long>(u) * kUnitRows + r;
+        x[j] = i < n && v < V ? __ldg(W + (v * H + static_cast<long long>(kb) * kBlockK) / 8 + c)
+                              : make_uint4(0u, 0u, 0u, 0u);
+        if (gw && i < n) x[j] = scale_chunk(x[j], gw + kb * kBlockK + c * 8);
+      }
+#pragma unroll
+      for (int j = 0; j < kVecs; ++j) {
+        const int i = i0 + j * blockDim.x;
+        if (i < n) out[(d.base + (i >> 6) * d.stride) / 16 + (i & 63)] = x[j];
+      }
+    }
   }
+}
+
+// CTA owning unit u when `units` units are split over G CTAs (unit_begin).
+__device__ __forceinline__ int unit_owner(int u, int units, int G) {
+  int c = static_cast<int>((static_cast<long long>(u) * G) / units);
+  while (c + 1 < G && unit_begin(c + 1, units, G) <= u) ++c;
+  while (c > 0 && unit_begin(c, units, G) > u) --c;
+  return c;
+}
+
+// For lm_head_softmax_kernel on G CTAs and groups of up to gmax tiles.
+__global__ void pack_weight_kernel(const uint4* __restrict__ W, uint4* __restrict__ out, int V,
+                                   int H, int units, int G, int gmax,
+                                   const __nv_bfloat16* __restrict__ gw) {
+  pack_units(W, out, V, H, units, gw, [=](int u) {
+    const CtaPlan pl = cta_plan(unit_owner(u, units, G), units, G, gmax);
+    const int row = (u - pl.u0) * kUnitRows;  // in the CTA's rows
+    const int t = row / kRowsPerTile, g = t / pl.gsz;
+    return PackDst{static_cast<long long>(pl.stage_offset(g, 0, t, H)) +
+                       (row - t * kRowsPerTile) * 128,
+                   static_cast<long long>(pl.group_rows(g)) * 128};
+  });
 }
 
 // Wait used only on the abort path, for copies this CTA already issued.

@@ -199,36 +199,25 @@ __host__ __device__ inline size_t pair_smem_bytes(int n_stages, bool swap) {
          static_cast<size_t>(2 * kPairMaxRing + 9) * 8 + 16 + 3 * kPairHalf * 4;
 }
 
-// Pack W [V, H] (row-major bf16) for the pair kernel in blocks of `run` rows x
-// 64 columns, the K blocks of a run one after the other; each row's 128 bytes
-// with the 128-byte swizzle of 8-row atoms (16-byte chunk c of row r at
-// c ^ (r & 7)); rows >= V zero.  The kernel reads it through a tensor map of
-// 64 columns with no swizzle: K block kb of row r (r / run = q) is map row
-// q run KB + kb run + r - q run.  Two runs are used (pair_w_run):
+// For the pair kernel: blocks of `run` rows x 64 columns, the K blocks of a run
+// one after the other, rows >= V of the last run zero.  The kernel reads it
+// through a tensor map of 64 columns with no swizzle: K block kb of row r (r /
+// run = q) is map row q run KB + kb run + r - q run.  Two runs are used
+// (pair_w_run):
 //   128, when every tile is 128 rows high: a tile's K blocks are contiguous;
 //   all round8(V) rows, otherwise: any run of 8-row atoms of a K block is one
 //   contiguous block, so steps of one row tile may cut V evenly (pair_even_rows)
 //   and wider ones in 128-row tiles.  Reading 128-row tiles in this order is
 //   0.6 % slower (152064 x 3584, M = 96: 169.2 us a step against 170.5).
 __global__ void pack_w_tiles_kernel(const uint4* __restrict__ W, uint4* __restrict__ out, int V,
-                                    int H, int run, long long n_chunks,
+                                    int H, int run, int units,
                                     const __nv_bfloat16* __restrict__ gw) {
-  const int KB = H / kPairBlockK;
-  const long long run_rows = static_cast<long long>(run) * KB;
-  for (long long d = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; d < n_chunks;
-       d += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long row = d >> 3;
-    const long long q = row / run_rows;
-    const long long rem = row - q * run_rows;
-    const int kb = static_cast<int>(rem / run);
-    const int r = static_cast<int>(rem - static_cast<long long>(kb) * run);
-    const long long v = q * run + r;
-    const int cl = static_cast<int>(d & 7) ^ (r & 7);
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    if (v < V) val = W[(v * H + static_cast<long long>(kb) * kPairBlockK) / 8 + cl];
-    if (gw) val = scale_chunk(val, gw + kb * kPairBlockK + cl * 8);
-    out[d] = val;
-  }
+  const long long KB = H / kPairBlockK;
+  pack_units(W, out, V, H, units, gw, [=](int u) {
+    const long long row = static_cast<long long>(u) * kUnitRows;
+    const long long q = row / run;
+    return PackDst{(q * run * KB + row - q * run) * 128, run * 128ll};
+  });
 }
 
 // Rows per run of the packed W, and its rows of 64 columns.

@@ -147,40 +147,21 @@ __host__ __device__ inline RowsPlan rows_plan(int c, int units, int G) {
   return p;
 }
 
-// Pack W [V, H] (row-major bf16) for lm_head_rows_kernel on G CTAs: CTA c's
-// groups in order, each group's K blocks in order, each K block the group's
-// rows in the 128-byte-swizzled K-major layout (row r's 16-byte chunk c at
-// r * 128 + (c ^ (r & 7)) * 16, 8-row atoms of 1 KiB).  Rows >= V are zero;
-// gw (bf16 [H], or null) is the final-norm weight folded in.  One thread per
-// destination 16-byte chunk; n_chunks = units * kUnitRows * H / 8.
+// For lm_head_rows_kernel on G CTAs: CTA c's groups in order, each group's K
+// blocks in order, each K block the group's rows.
 __global__ void pack_weight_rows_kernel(const uint4* __restrict__ W, uint4* __restrict__ out, int V,
-                                        int H, int units, int G, long long n_chunks,
+                                        int H, int units, int G,
                                         const __nv_bfloat16* __restrict__ gw) {
-  const long long unit_bytes = 2ll * kUnitRows * H;
-  for (long long d = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; d < n_chunks;
-       d += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long byte = d * 16;
-    const int u = static_cast<int>(byte / unit_bytes);
-    int c = static_cast<int>((static_cast<long long>(u) * G) / units);
-    while (c + 1 < G && unit_begin(c + 1, units, G) <= u) ++c;
-    while (c > 0 && unit_begin(c, units, G) > u) --c;
-    const RowsPlan pl = rows_plan(c, units, G);
+  pack_units(W, out, V, H, units, gw, [=](int u) {
+    const RowsPlan pl = rows_plan(unit_owner(u, units, G), units, G);
     // Group holding unit u (groups are whole units).
     int g = static_cast<int>((static_cast<long long>(u - pl.u0) * pl.n_groups) / (pl.u1 - pl.u0));
     while (g + 1 < pl.n_groups && pl.group_unit(g + 1) <= u - pl.u0) ++g;
     while (g > 0 && pl.group_unit(g) > u - pl.u0) --g;
-    const long long rem = byte - static_cast<long long>(pl.group_row0(g)) * 2 * H;
-    const int grow = pl.group_rows(g);
-    const int kb = static_cast<int>(rem / (grow * 128));
-    const int rem2 = static_cast<int>(rem - static_cast<long long>(kb) * grow * 128);
-    const int r = rem2 >> 7;
-    const int cl = ((rem2 >> 4) & 7) ^ (r & 7);
-    const long long v = static_cast<long long>(pl.group_row0(g)) + r;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    if (v < V) val = W[(v * H + static_cast<long long>(kb) * kBlockK) / 8 + cl];
-    if (gw) val = scale_chunk(val, gw + kb * kBlockK + cl * 8);
-    out[d] = val;
-  }
+    return PackDst{static_cast<long long>(pl.stage_offset(g, 0, H)) +
+                       (u - pl.u0 - pl.group_unit(g)) * (kUnitRows * 128),
+                   static_cast<long long>(pl.group_rows(g)) * 128};
+  });
 }
 
 // Single-kernel step only (p.fused = 1, p.M_fixed <= 128), W packed by
