@@ -300,6 +300,7 @@ struct cai_ctx {
   bool shard_first = false;    // ... and it was the block's step zero
   int G = 0, n_stages = 0, n_bslots = 0, n_max = 0, slot_cols = 0, gmax = 1, tmem_cols = 0;
   int b_slot_bytes = 0;
+  int w_stage = 0;  // rows-operand head: bytes of a W stage
   size_t head_smem = 0;
   int blk = 0, t_next = 0;
   int64_t last_step_id = -1;
@@ -671,6 +672,7 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
   hp.units = (cfg.V + kUnitRows - 1) / kUnitRows;
   hp.n_stages = c->n_stages;
   hp.n_bslots = c->n_bslots;
+  hp.w_stage = c->w_stage;
   hp.b_slot_bytes = c->b_slot_bytes;
   hp.slot_cols = c->slot_cols;
   hp.gmax = c->gmax;
@@ -904,21 +906,28 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
       return CAI_ERR_CUDA;
     }
     const size_t rlimit = static_cast<size_t>(smem_optin) - ra.sharedSizeBytes;
-    // As many W stages as fit next to a rows ring of the same depth (the
-    // rows stages are small); CAI_ROWS_STAGES caps the W ring (tuning knob).
-    // Four 32 KiB W stages in flight per SM: deeper rings stream faster on
-    // most SMs but starve some (measured, LLaDA shape: finish spread 4 us at
-    // 4 stages, 20 us at 6), and a step waits for its slowest CTA.
+    // kRowsInFlight bytes of W in stages of the largest group's size;
+    // CAI_ROWS_STAGES sets the ring's depth (tuning knob).
+    int most = 0;
+    for (int cta = 0; cta < c->G; ++cta) {
+      const RowsPlan pl = rows_plan(cta, units, c->G);
+      for (int g = 0; g < pl.n_groups; ++g) most = pl.group_rows(g) > most ? pl.group_rows(g) : most;
+    }
+    // The MMA reads round16(rows) rows of a W stage, and 128 rows from the last
+    // rows part on, into the W ring (two stages at least), which also holds the
+    // commit's working set once it is drained.
+    static_assert(sizeof(CommitSmem) <= 2 * 64 * 128, "the smallest W ring holds it");
+    const int ws = (most < 64 ? 64 : round_up(most, 16)) * 128;
     const int hs = rows_h_stride(c->BP);
     const int scap2 = env_int("CAI_ROWS_STAGES");
-    int st = scap2 >= 2 && scap2 <= 8 ? scap2 : 4;
-    while (st > 2 && rows_smem_bytes(st, 2 * st, hs) > rlimit) --st;
-    int bs = 2 * st;
-    while (bs > 2 && rows_smem_bytes(st, bs, hs) > rlimit) --bs;
+    int st = cfg->H >= 2048 && kRowsInFlight / ws >= 5 ? 5 : 4;
+    if (scap2 >= 2 && scap2 <= 8) st = scap2;
+    while (st > 2 && rows_smem_bytes(st, ws, hs) > rlimit) --st;
+    c->w_stage = ws;
     c->n_stages = st;
-    c->n_bslots = bs;
+    c->n_bslots = st;
     c->tmem_cols = kRowsTmemCols;
-    c->head_smem = rows_smem_bytes(st, bs, hs);
+    c->head_smem = rows_smem_bytes(st, ws, hs);
   }
 
   // Pair kernel launch shape: a persistent grid of as many 2-CTA clusters as

@@ -17,13 +17,14 @@
 //
 // Rows stages.  The MMA reads 128 rows of A, but only the first mq =
 // round16(M) are the step's; the accumulator rows past M are never read.  So
-// a rows stage owns only mq rows (the stride between stages is mq * 128 bytes
-// rounded up to 1 KiB, 4 KiB for M <= 32) and the MMA's read of the other
-// rows runs on into the following stages (and, for the last ones, the W ring
-// placed after them): whatever it finds there only reaches accumulator rows
-// that no thread loads.  Small stages let the rows ring be as deep as the W
-// ring, so the producer, which issues both, never holds back a W copy for
-// want of a rows stage.
+// the rows part of a stage owns only mq rows (the parts lie mq * 128 bytes
+// rounded up to 1 KiB apart, 4 KiB for M <= 32, before the W parts) and the
+// MMA's read of the other rows runs on into the following parts (and, for the
+// last ones, the W ring): whatever it finds there only reaches accumulator rows
+// that no thread loads.  A stage's rows and W complete one barrier and are
+// freed by one commit; with a ring and barriers of their own for the rows a
+// stage took two waits and two commits: 1024 x 22000 11.3 us a step, now 10.0;
+// 2048 x 50003 30.0, now 27.1; 4096 x 126464 with 128 rows 141.8, now 134.2.
 //
 // Work split: as lm_head_softmax_kernel, V in units of 8 rows over the CTAs;
 // a CTA's rows form equal groups of at most 256 vocabulary rows (RowsPlan),
@@ -58,7 +59,7 @@ namespace cai {
 
 constexpr int kRowsM = 128;                          // MMA M: rows of the step, padded
 constexpr int kRowsGroupRows = 256;                  // MMA N: vocabulary rows per group
-constexpr int kRowsWStage = kRowsGroupRows * 128;    // 32 KiB: one K block of a group
+constexpr int kRowsWStage = kRowsGroupRows * 128;    // 32 KiB: one K block of the largest group
 constexpr int kRowsHStageMax = kRowsM * 128;         // 16 KiB: all 128 rows of a K block
 constexpr int kRowsTmemCols = 2 * kRowsGroupRows;    // two accumulators
 constexpr int kRowsEpiWarps = 8;                     // two per tensor-memory quarter
@@ -71,19 +72,16 @@ __host__ __device__ inline int rows_h_stride(int M) {
 
 // The rows ring comes first, then the W ring, whose first 12 KiB or more
 // cover the last rows stage's read past its own bytes.
-__host__ __device__ inline size_t rows_smem_bytes(int n_stages, int n_bslots, int h_stride) {
-  return 1024 + static_cast<size_t>(n_bslots) * h_stride +
-         static_cast<size_t>(n_stages) * kRowsWStage +
-         static_cast<size_t>(2 * n_stages + 2 * n_bslots + 6) * 8 + 16;
+__host__ __device__ inline size_t rows_smem_bytes(int n_stages, int w_stage, int h_stride) {
+  return 1024 + static_cast<size_t>(n_stages) * (h_stride + w_stage) +
+         static_cast<size_t>(2 * n_stages + 6) * 8 + 16;
 }
 
 struct RowsSmem {
-  uint8_t* h;         // n_bslots x h_stride
-  uint8_t* w;         // n_stages x 32 KiB
-  uint64_t* full_w;   // n_stages
-  uint64_t* empty_w;  // n_stages
-  uint64_t* full_h;   // n_bslots
-  uint64_t* empty_h;  // n_bslots
+  uint8_t* h;         // n_stages x h_stride
+  uint8_t* w;         // n_stages x w_stage
+  uint64_t* full;     // n_stages: the stage's W and rows landed
+  uint64_t* empty;    // n_stages: the MMAs are done with the stage
   uint64_t* accf;     // 2: accumulator ready
   uint64_t* acce;     // 2: accumulator drained by the epilogue warps
   uint64_t* drain;    // 1
@@ -93,18 +91,16 @@ struct RowsSmem {
   volatile int* skip;
 };
 
-__device__ __forceinline__ RowsSmem rows_carve(uint8_t* raw, int n_stages, int n_bslots,
+__device__ __forceinline__ RowsSmem rows_carve(uint8_t* raw, int n_stages, int w_stage,
                                                int h_stride) {
   RowsSmem s;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   s.h = base;
-  s.w = s.h + static_cast<size_t>(n_bslots) * h_stride;
-  s.full_w = reinterpret_cast<uint64_t*>(s.w + static_cast<size_t>(n_stages) * kRowsWStage);
-  s.empty_w = s.full_w + n_stages;
-  s.full_h = s.empty_w + n_stages;
-  s.empty_h = s.full_h + n_bslots;
-  s.accf = s.empty_h + n_bslots;
+  s.w = s.h + static_cast<size_t>(n_stages) * h_stride;
+  s.full = reinterpret_cast<uint64_t*>(s.w + static_cast<size_t>(n_stages) * w_stage);
+  s.empty = s.full + n_stages;
+  s.accf = s.empty + n_stages;
   s.acce = s.accf + 2;
   s.drain = s.acce + 2;
   s.xch = s.drain + 1;
@@ -139,6 +135,14 @@ struct RowsPlan {
   }
 };
 
+// W stages: 128 KiB of weight in flight per SM, at least four stages and with a
+// long K five.  Deeper rings stream faster on most SMs but starve some (LLaDA
+// shape: finish spread 4 us at four 27 KiB stages, 20 us at six), and a step
+// waits for its slowest CTA; a short K pays for filling a deeper ring (1024 x
+// 40000: 17.3 us a step at four stages, 18.3 at eight; 3584 x 80000: 77.1 at
+// four, 75.0 at five, 75.1 at eight).
+constexpr int kRowsInFlight = 128 << 10;
+
 __host__ __device__ inline RowsPlan rows_plan(int c, int units, int G) {
   RowsPlan p;
   p.u0 = unit_begin(c, units, G);
@@ -165,7 +169,7 @@ __global__ void pack_weight_rows_kernel(const uint4* __restrict__ W, uint4* __re
 }
 
 // Single-kernel step only (p.fused = 1, p.M_fixed <= 128), W packed by
-// pack_weight_rows_kernel.  p.n_stages is the W ring depth (32 KiB stages),
+// pack_weight_rows_kernel.  p.n_stages is the W ring depth (p.w_stage bytes each),
 // p.n_bslots the rows ring depth (stages rows_h_stride(M) apart).  kNorm: row
 // r's logits are scaled by 1 / sqrt(mean h^2 + eps) of the row, which the
 // epilogue warps compute from the step's rows (p.hid).
@@ -176,7 +180,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int h_stride = rows_h_stride(p.M_fixed);
-  RowsSmem sm = rows_carve(smem_raw, p.n_stages, p.n_bslots, h_stride);
+  RowsSmem sm = rows_carve(smem_raw, p.n_stages, p.w_stage, h_stride);
   const int cta = blockIdx.x;
   const RowsPlan pl = rows_plan(cta, p.units, gridDim.x);
   const int KB = p.H / kBlockK;
@@ -187,12 +191,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.n_stages; ++s) {
-      mbar_init(&sm.full_w[s], 1);
-      mbar_init(&sm.empty_w[s], 1);
-    }
-    for (int s = 0; s < p.n_bslots; ++s) {
-      mbar_init(&sm.full_h[s], 1);
-      mbar_init(&sm.empty_h[s], 1);
+      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.empty[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&sm.accf[a], 1);
@@ -210,9 +210,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     for (int g = 0; g < pl.n_groups && i < n_pre; ++g)
       for (int kb = 0; kb < KB && i < n_pre; ++kb, ++i) {
         const uint32_t bytes = static_cast<uint32_t>(pl.group_rows(g) * 128);
-        mbar_expect_tx(&sm.full_w[i], bytes);
-        bulk_load(sm.w + static_cast<size_t>(i) * kRowsWStage,
-                  p.wpk + pl.stage_offset(g, kb, p.H), bytes, &sm.full_w[i], pol_w);
+        mbar_expect_tx(&sm.full[i], bytes);
+        bulk_load(sm.w + static_cast<size_t>(i) * p.w_stage,
+                  p.wpk + pl.stage_offset(g, kb, p.H), bytes, &sm.full[i], pol_w);
       }
   }
   grid_launch_dependents();  // every thread: the CTA counts once all of them have
@@ -235,8 +235,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     const uint64_t pol_w = policy_evict_first();
     const uint64_t pol_h = policy_evict_last();
     const bool leader = elect_one();
-    Ring rw, rh;
-    int w_issued = 0, h_issued = 0;
+    Ring r;
+    int issued = 0;
     bool ok = true, decided = !spec;
     // Rows copied from the host on the context's side stream: wait (bounded)
     // for that copy's sequence word before the first row load.
@@ -250,60 +250,48 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
       const uint32_t wbytes = static_cast<uint32_t>(pl.group_rows(g) * 128);
       const uint8_t* wsrc = p.wpk + pl.stage_offset(g, 0, p.H);
       for (int kb = 0; kb < KB; ++kb) {
-        ok = ok && mbar_wait(&sm.empty_h[rh.slot], rh.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
+        ok = ok && mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
         if (!decided &&
             previous_left_nothing(__shfl_sync(0xffffffffu, pub_w, 0), p.cp.step_id, decided)) {
-          // Stop: the rows stage completes empty and carries the stop mark,
+          // Stop: the stage completes without rows and carries the stop mark,
           // this K block's number, to the MMA warp, which consumes every
           // stage issued before it first (no copy may be in flight when the
           // CTA leaves or its shared memory is used for the commit).
           if (leader && ok) {
             *sm.skip = g * KB + kb + 1;
-            mbar_arrive(&sm.full_h[rh.slot]);
+            mbar_arrive(&sm.full[r.slot]);
           }
+          issued += ok ? 1 : 0;
           g = pl.n_groups;
           break;
         }
         if (!decided) pub_w = load_pub(p.cp.pub);
         if (leader && ok) {
-          mbar_arrive_expect_tx(&sm.full_h[rh.slot], static_cast<uint32_t>(mq * 128));
-          tma_load_2d(sm.h + rh.slot * h_stride, &tm_h, &sm.full_h[rh.slot], kb * kBlockK, 0, pol_h);
-        }
-        h_issued += ok ? 1 : 0;
-        rh.next(p.n_bslots);
-        if (w_issued < n_pre) {
-          if (leader && ok) mbar_arrive(&sm.full_w[rw.slot]);  // copy already in flight
-        } else {
-          ok = ok && mbar_wait(&sm.empty_w[rw.slot], rw.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
-          if (leader && ok) {
-            mbar_arrive_expect_tx(&sm.full_w[rw.slot], wbytes);
-            bulk_load(sm.w + rw.slot * kRowsWStage, wsrc + static_cast<size_t>(kb) * wbytes, wbytes,
-                      &sm.full_w[rw.slot], pol_w);
-          }
+          const bool pre = issued < n_pre;  // the W copy is already in flight
+          mbar_arrive_expect_tx(&sm.full[r.slot],
+                                static_cast<uint32_t>(mq * 128) + (pre ? 0u : wbytes));
+          tma_load_2d(sm.h + r.slot * h_stride, &tm_h, &sm.full[r.slot], kb * kBlockK, 0, pol_h);
+          if (!pre)
+            bulk_load(sm.w + r.slot * p.w_stage, wsrc + static_cast<size_t>(kb) * wbytes, wbytes,
+                      &sm.full[r.slot], pol_w);
         }
         __syncwarp();
-        w_issued += ok ? 1 : 0;
-        rw.next(p.n_stages);
+        issued += ok ? 1 : 0;
+        r.next(p.n_stages);
       }
       ok = __all_sync(0xffffffffu, ok);
     }
     if (leader) {
-      if (w_issued < n_pre) {
+      if (issued < n_pre) {
         // A stop or an abort before the prefetched stages were claimed:
         // complete their phases so the copies can drain.
-        for (int i = w_issued; i < n_pre; ++i) mbar_arrive(&sm.full_w[i]);
-        for (int i = w_issued; i < n_pre; ++i) mbar_drain(&sm.full_w[i], 0, p.err);
+        for (int i = issued; i < n_pre; ++i) mbar_arrive(&sm.full[i]);
+        for (int i = issued; i < n_pre; ++i) mbar_drain(&sm.full[i], 0, p.err);
       }
       if (!ok) {
         // Abort path: let the copies already in flight land before exit.
-        const int fw = w_issued > p.n_stages ? w_issued - p.n_stages : 0;
-        for (int i = fw; i < w_issued; ++i)
-          mbar_drain(&sm.full_w[i % p.n_stages], static_cast<uint32_t>((i / p.n_stages) & 1),
-                     p.err);
-        const int fh = h_issued > p.n_bslots ? h_issued - p.n_bslots : 0;
-        for (int i = fh; i < h_issued; ++i)
-          mbar_drain(&sm.full_h[i % p.n_bslots], static_cast<uint32_t>((i / p.n_bslots) & 1),
-                     p.err);
+        for (int i = issued > p.n_stages ? issued - p.n_stages : 0; i < issued; ++i)
+          mbar_drain(&sm.full[i % p.n_stages], static_cast<uint32_t>((i / p.n_stages) & 1), p.err);
       }
     }
     __syncwarp();
@@ -313,7 +301,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     const bool leader = elect_one();
     const uint64_t h_desc = sdesc_k_sw128(smem_addr(sm.h));
     const uint64_t w_desc = sdesc_k_sw128(smem_addr(sm.w));
-    Ring rw, rh, racc;
+    Ring r, racc;
     bool ok = true, skipped = false;
     for (int g = 0; g < pl.n_groups && ok && !skipped; ++g) {
       const uint32_t n = static_cast<uint32_t>((pl.group_rows(g) + 15) & ~15);
@@ -324,25 +312,22 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(racc.slot * kRowsGroupRows);
       for (int kb = 0; kb < KB; ++kb) {
-        ok = ok && mbar_wait(&sm.full_h[rh.slot], rh.phase, sm.abort, p.err, kErrWaitFull);
+        ok = ok && mbar_wait(&sm.full[r.slot], r.phase, sm.abort, p.err, kErrWaitFull);
         if (spec && __any_sync(0xffffffffu, ok && *sm.skip == g * KB + kb + 1)) {
           skipped = true;
           break;
         }
-        ok = ok && mbar_wait(&sm.full_w[rw.slot], rw.phase, sm.abort, p.err, kErrWaitFull);
         tc_fence_after();
-        const uint64_t a = h_desc + static_cast<uint32_t>(rh.slot * h_stride >> 4);
-        const uint64_t b = w_desc + static_cast<uint32_t>(rw.slot * (kRowsWStage >> 4));
+        const uint64_t a = h_desc + static_cast<uint32_t>(r.slot * h_stride >> 4);
+        const uint64_t b = w_desc + static_cast<uint32_t>(r.slot * p.w_stage >> 4);
         if (leader && ok) {
 #pragma unroll
           for (int kk = 0; kk < kBlockK / 16; ++kk)
             mma_bf16(d_tmem, a + 2 * kk, b + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-          mma_commit(&sm.empty_w[rw.slot]);
-          mma_commit(&sm.empty_h[rh.slot]);
+          mma_commit(&sm.empty[r.slot]);
         }
         __syncwarp();
-        rw.next(p.n_stages);
-        rh.next(p.n_bslots);
+        r.next(p.n_stages);
       }
       ok = __all_sync(0xffffffffu, ok);
       if (!ok || skipped) break;
