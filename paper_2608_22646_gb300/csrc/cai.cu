@@ -300,7 +300,8 @@ struct cai_ctx {
   bool shard_first = false;    // ... and it was the block's step zero
   int G = 0, n_stages = 0, n_bslots = 0, n_max = 0, slot_cols = 0, gmax = 1, tmem_cols = 0;
   int b_slot_bytes = 0;
-  int w_stage = 0;  // rows-operand head: bytes of a W stage
+  int w_stage = 0;  // rows-operand head: bytes of a stage's W, and ...
+  int kps = 1;      // ... K blocks per stage
   size_t head_smem = 0;
   int blk = 0, t_next = 0;
   int64_t last_step_id = -1;
@@ -673,6 +674,7 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
   hp.n_stages = c->n_stages;
   hp.n_bslots = c->n_bslots;
   hp.w_stage = c->w_stage;
+  hp.kps = c->kps;
   hp.b_slot_bytes = c->b_slot_bytes;
   hp.slot_cols = c->slot_cols;
   hp.gmax = c->gmax;
@@ -917,10 +919,13 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     // rows part on, into the W ring (two stages at least), which also holds the
     // commit's working set once it is drained.
     static_assert(sizeof(CommitSmem) <= 2 * 64 * 128, "the smallest W ring holds it");
-    const int ws = (most < 64 ? 64 : round_up(most, 16)) * 128;
-    const int hs = rows_h_stride(c->BP);
+    int ws = (most < 64 ? 64 : round_up(most, 16)) * 128;
+    int hs = rows_h_stride(c->BP);
     const int scap2 = env_int("CAI_ROWS_STAGES");
-    int st = cfg->H >= 2048 && kRowsInFlight / ws >= 5 ? 5 : 4;
+    c->kps = rows_k_blocks(cfg->V, cfg->H, ws, hs, rlimit);
+    int st = c->kps == 1 && cfg->H >= 2048 && kRowsInFlight / ws >= 5 ? 5 : 4;
+    ws *= c->kps;
+    hs *= c->kps;
     if (scap2 >= 2 && scap2 <= 8) st = scap2;
     while (st > 2 && rows_smem_bytes(st, ws, hs) > rlimit) --st;
     c->w_stage = ws;

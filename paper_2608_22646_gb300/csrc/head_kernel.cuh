@@ -88,7 +88,8 @@ struct HeadParams {
   int units;           // ceil(V / kUnitRows)
   int n_stages;        // depth of the W ring (16 KiB slots)
   int n_bslots;        // depth of the hidden-state ring
-  int w_stage;         // rows-operand kernel: bytes of a W stage
+  int w_stage;         // rows-operand kernel: bytes of a stage's W,
+  int kps;             // K blocks per stage (1 or 2)
   int b_slot_bytes;    // n_max * 128
   int slot_cols;       // tensor-memory columns per tile accumulator (round32(n_max))
   int gmax;            // largest tile group

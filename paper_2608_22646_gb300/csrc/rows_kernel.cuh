@@ -17,7 +17,7 @@
 //
 // Rows stages.  The MMA reads 128 rows of A, but only the first mq =
 // round16(M) are the step's; the accumulator rows past M are never read.  So
-// the rows part of a stage owns only mq rows (the parts lie mq * 128 bytes
+// the rows part of a K block owns only mq rows (the parts lie mq * 128 bytes
 // rounded up to 1 KiB apart, 4 KiB for M <= 32, before the W parts) and the
 // MMA's read of the other rows runs on into the following parts (and, for the
 // last ones, the W ring): whatever it finds there only reaches accumulator rows
@@ -72,8 +72,8 @@ __host__ __device__ inline int rows_h_stride(int M) {
 
 // The rows ring comes first, then the W ring, whose first 12 KiB or more
 // cover the last rows stage's read past its own bytes.
-__host__ __device__ inline size_t rows_smem_bytes(int n_stages, int w_stage, int h_stride) {
-  return 1024 + static_cast<size_t>(n_stages) * (h_stride + w_stage) +
+__host__ __device__ inline size_t rows_smem_bytes(int n_stages, int w_stage, int h_stage) {
+  return 1024 + static_cast<size_t>(n_stages) * (h_stage + w_stage) +
          static_cast<size_t>(2 * n_stages + 6) * 8 + 16;
 }
 
@@ -92,12 +92,12 @@ struct RowsSmem {
 };
 
 __device__ __forceinline__ RowsSmem rows_carve(uint8_t* raw, int n_stages, int w_stage,
-                                               int h_stride) {
+                                               int h_stage) {
   RowsSmem s;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   s.h = base;
-  s.w = s.h + static_cast<size_t>(n_stages) * h_stride;
+  s.w = s.h + static_cast<size_t>(n_stages) * h_stage;
   s.full = reinterpret_cast<uint64_t*>(s.w + static_cast<size_t>(n_stages) * w_stage);
   s.empty = s.full + n_stages;
   s.accf = s.empty + n_stages;
@@ -135,13 +135,26 @@ struct RowsPlan {
   }
 };
 
-// W stages: 128 KiB of weight in flight per SM, at least four stages and with a
-// long K five.  Deeper rings stream faster on most SMs but starve some (LLaDA
+// W stages of one K block: at least four, and with a long K five while about
+// 128 KiB of weight are in flight per SM.  Deeper rings stream faster on most SMs but starve some (LLaDA
 // shape: finish spread 4 us at four 27 KiB stages, 20 us at six), and a step
 // waits for its slowest CTA; a short K pays for filling a deeper ring (1024 x
 // 40000: 17.3 us a step at four stages, 18.3 at eight; 3584 x 80000: 77.1 at
 // four, 75.0 at five, 75.1 at eight).
 constexpr int kRowsInFlight = 128 << 10;
+
+// K blocks per stage, given the bytes of one block's W and rows parts: two
+// where four such stages fit, or three and the weight stays in L2.  A stage's
+// waits, commit and copies take ~0.25 us whatever it holds, which bounds
+// weights that come from L2 (1024 x 10000 9.0 -> 7.8 us a step, 1024 x 40000 15.4
+// -> 13.3, 2048 x 50003 27.4 -> 24.6).  At the memory's rate it makes no
+// difference back to back, but three stages of 64 KiB start a lone step later
+// (3584 x 152064 161.8 -> 164.6 us), and with two in flight the stream stalls
+// (4096 x 126464, 128 rows: 136.4 -> 143).
+__host__ inline int rows_k_blocks(int V, int H, int w_bytes, int h_bytes, size_t smem_limit) {
+  const int need = 2ll * V * H <= 128ll << 20 ? 3 : 4;
+  return H >= 2 * kBlockK && rows_smem_bytes(need, 2 * w_bytes, 2 * h_bytes) <= smem_limit ? 2 : 1;
+}
 
 __host__ __device__ inline RowsPlan rows_plan(int c, int units, int G) {
   RowsPlan p;
@@ -180,14 +193,14 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int h_stride = rows_h_stride(p.M_fixed);
-  RowsSmem sm = rows_carve(smem_raw, p.n_stages, p.w_stage, h_stride);
+  RowsSmem sm = rows_carve(smem_raw, p.n_stages, p.w_stage, p.kps * h_stride);
   const int cta = blockIdx.x;
   const RowsPlan pl = rows_plan(cta, p.units, gridDim.x);
   const int KB = p.H / kBlockK;
   const int M = p.M_fixed;
   const int mq = (M + 15) & ~15;  // rows loaded per K block (TMA fills rows past B P with zeros)
   const bool spec = !p.first;     // may find out that nothing is masked
-  const int n_pre = p.prefetch ? min(p.n_stages, pl.n_groups * KB) : 0;
+  const int n_pre = p.prefetch ? min(p.n_stages, pl.n_groups * ((KB + p.kps - 1) / p.kps)) : 0;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.n_stages; ++s) {
@@ -208,8 +221,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     const uint64_t pol_w = policy_evict_first();
     int i = 0;
     for (int g = 0; g < pl.n_groups && i < n_pre; ++g)
-      for (int kb = 0; kb < KB && i < n_pre; ++kb, ++i) {
-        const uint32_t bytes = static_cast<uint32_t>(pl.group_rows(g) * 128);
+      for (int kb = 0; kb < KB && i < n_pre; kb += p.kps, ++i) {
+        const uint32_t bytes = static_cast<uint32_t>(pl.group_rows(g) * 128 * min(p.kps, KB - kb));
         mbar_expect_tx(&sm.full[i], bytes);
         bulk_load(sm.w + static_cast<size_t>(i) * p.w_stage,
                   p.wpk + pl.stage_offset(g, kb, p.H), bytes, &sm.full[i], pol_w);
@@ -249,7 +262,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     for (int g = 0; g < pl.n_groups && ok; ++g) {
       const uint32_t wbytes = static_cast<uint32_t>(pl.group_rows(g) * 128);
       const uint8_t* wsrc = p.wpk + pl.stage_offset(g, 0, p.H);
-      for (int kb = 0; kb < KB; ++kb) {
+      for (int kb = 0; kb < KB; kb += p.kps) {
         ok = ok && mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
         if (!decided &&
             previous_left_nothing(__shfl_sync(0xffffffffu, pub_w, 0), p.cp.step_id, decided)) {
@@ -268,12 +281,16 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
         if (!decided) pub_w = load_pub(p.cp.pub);
         if (leader && ok) {
           const bool pre = issued < n_pre;  // the W copy is already in flight
-          mbar_arrive_expect_tx(&sm.full[r.slot],
-                                static_cast<uint32_t>(mq * 128) + (pre ? 0u : wbytes));
-          tma_load_2d(sm.h + r.slot * h_stride, &tm_h, &sm.full[r.slot], kb * kBlockK, 0, pol_h);
+          const uint32_t nk = static_cast<uint32_t>(min(p.kps, KB - kb));
+          mbar_arrive_expect_tx(&sm.full[r.slot], nk * (static_cast<uint32_t>(mq * 128) +
+                                                        (pre ? 0u : wbytes)));
+          uint8_t* h = sm.h + r.slot * p.kps * h_stride;
+          tma_load_2d(h, &tm_h, &sm.full[r.slot], kb * kBlockK, 0, pol_h);
+          if (nk > 1)
+            tma_load_2d(h + h_stride, &tm_h, &sm.full[r.slot], (kb + 1) * kBlockK, 0, pol_h);
           if (!pre)
-            bulk_load(sm.w + r.slot * p.w_stage, wsrc + static_cast<size_t>(kb) * wbytes, wbytes,
-                      &sm.full[r.slot], pol_w);
+            bulk_load(sm.w + r.slot * p.w_stage, wsrc + static_cast<size_t>(kb) * wbytes,
+                      nk * wbytes, &sm.full[r.slot], pol_w);
         }
         __syncwarp();
         issued += ok ? 1 : 0;
@@ -311,19 +328,26 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
       if (!ok) break;
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(racc.slot * kRowsGroupRows);
-      for (int kb = 0; kb < KB; ++kb) {
+      const uint32_t w_next = static_cast<uint32_t>(pl.group_rows(g) * 128) >> 4;
+      for (int kb = 0; kb < KB; kb += p.kps) {
         ok = ok && mbar_wait(&sm.full[r.slot], r.phase, sm.abort, p.err, kErrWaitFull);
         if (spec && __any_sync(0xffffffffu, ok && *sm.skip == g * KB + kb + 1)) {
           skipped = true;
           break;
         }
         tc_fence_after();
-        const uint64_t a = h_desc + static_cast<uint32_t>(r.slot * h_stride >> 4);
+        const uint64_t a = h_desc + static_cast<uint32_t>(r.slot * p.kps * h_stride >> 4);
         const uint64_t b = w_desc + static_cast<uint32_t>(r.slot * p.w_stage >> 4);
         if (leader && ok) {
 #pragma unroll
           for (int kk = 0; kk < kBlockK / 16; ++kk)
             mma_bf16(d_tmem, a + 2 * kk, b + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+          if (kb + 1 < KB && p.kps > 1) {
+            const uint64_t a1 = a + static_cast<uint32_t>(h_stride >> 4), b1 = b + w_next;
+#pragma unroll
+            for (int kk = 0; kk < kBlockK / 16; ++kk)
+              mma_bf16(d_tmem, a1 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+          }
           mma_commit(&sm.empty[r.slot]);
         }
         __syncwarp();
