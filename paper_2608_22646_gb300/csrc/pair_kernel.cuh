@@ -102,6 +102,7 @@ constexpr int kPairBlockK = 64;       // K per stage (one 128-byte swizzled row)
 constexpr int kPairHalfBytes = kPairHalf * kPairBlockK * 2;  // 16 KiB
 constexpr int kPairStageBytes = 2 * kPairHalfBytes;          // A half + B half
 constexpr int kPairTmemCols = 2 * kPairTileVocab;            // two accumulators
+constexpr int kSwapTwoBlocks = 96;  // swapped tiles up to this wide: two K blocks per stage
 constexpr int kSwapColStep = 32;    // swapped orientation: granularity of N
 constexpr int kSwapXchBytes = 2 * 4 * kPairTileVocab * 16;  // cross-warp exchange, two buffers
 constexpr int kSwapChunks = kPairTileVocab / 32;  // most 16-column chunks of an epilogue warp
@@ -365,8 +366,14 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
   // ring (n_stages slots of kPairStageBytes) is re-cut to that size: more
   // stages in flight for narrower tiles.  Unswapped steps do not use the
   // swapped epilogue's exchange buffer, which follows the ring: one more stage.
-  const int stage_stride =
-      swap ? kPairHalfBytes + (rt_rows / 2) * kPairBlockK * 2 : kPairStageBytes;
+  // K blocks per stage.  Two halve the waits and commits, which bounds narrow
+  // tiles of weights that come from L2; only the allocation-free head has them:
+  // it also runs blocks of up to 128 rows on this kernel (1088 x 31560, 32 rows
+  // 13.5 -> 11.8 us a call, 4096 x 126464 153.0 -> 150.3), while in a context the
+  // longer loop cost steps of two row tiles 1.6 %.
+  const int kps = kStatic && swap && rt_rows <= kSwapTwoBlocks ? 2 : 1;
+  const int rows_bytes = (swap ? rt_rows / 2 : kPairHalf) * kPairBlockK * 2;
+  const int stage_stride = kps * (kPairHalfBytes + rows_bytes);
   const int ring_bytes =
       p.n_stages * kPairStageBytes + (!swap && p.swap_max_n > 0 ? kSwapXchBytes : 0);
   const int n_ring = min(p.ring_max, ring_bytes / stage_stride);
@@ -392,18 +399,27 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
       // First row of this CTA's half of the tile's rows.
       const int a_row = j * rt_rows + static_cast<int>(rank) * (swap ? rt_rows / 2 : kPairHalf);
       const int w_row = (2 * v + static_cast<int>(rank)) * th;
-      for (int kb = 0; kb < KB; ++kb) {
+      for (int kb = 0; kb < KB; kb += kps) {
         ok = ok && mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
         if (leader && ok) {
           uint8_t* dst = sm.stage + static_cast<size_t>(r.slot) * stage_stride;
           const uint32_t bar = full0 + static_cast<uint32_t>(r.slot * 8);
           // The even CTA arms the stage for the bytes of both CTAs; a copy of
           // the odd CTA that completes first leaves the phase open until then.
-          if (rank == 0) mbar_arrive_expect_tx(&sm.full[r.slot], stage_tx);
+          const bool two = kb + 1 < KB && kps > 1;
+          if (rank == 0) mbar_arrive_expect_tx(&sm.full[r.slot], two ? 2 * stage_tx : stage_tx);
           if (swap) {
-            // A: the W half; B: the CTA's rows, one box of box_rows.
+            // A: the W half; B: the CTA's rows, one box of box_rows.  (Two K
+            // blocks: W, W, rows, rows.)
+            uint8_t* rows = dst + kps * kPairHalfBytes;
             tma_load_2d_pair_nohint(dst, tmw, bar, kb * p.w_dx, w_row * p.w_ry + kb * p.w_dy);
-            tma_load_2d_pair(dst + kPairHalfBytes, &hm.box[q1], bar, kb * kPairBlockK, a_row, pol_a);
+            if (two)
+              tma_load_2d_pair_nohint(dst + kPairHalfBytes, tmw, bar, (kb + 1) * p.w_dx,
+                                      w_row * p.w_ry + (kb + 1) * p.w_dy);
+            tma_load_2d_pair(rows, &hm.box[q1], bar, kb * kPairBlockK, a_row, pol_a);
+            if (two)
+              tma_load_2d_pair(rows + rows_bytes, &hm.box[q1], bar, (kb + 1) * kPairBlockK, a_row,
+                               pol_a);
           } else {
             tma_load_2d_pair(dst, &tm_a, bar, kb * kPairBlockK, a_row, pol_a);
             tma_load_2d_pair_nohint(dst + kPairHalfBytes, tmw, bar, kb * p.w_dx,
@@ -439,15 +455,22 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kPairTileVocab);
-        for (int kb = 0; kb < KB; ++kb) {
+        for (int kb = 0; kb < KB; kb += kps) {
           ok = ok && mbar_wait_cluster(&sm.full[r.slot], r.phase, sm.abort, p.err, kErrWaitFull);
           tc_fence_after();
           const uint64_t a = desc0 + static_cast<uint32_t>(r.slot * stage_stride >> 4);
-          const uint64_t b = a + (kPairHalfBytes >> 4);
+          const uint64_t b = a + static_cast<uint32_t>(kps * kPairHalfBytes >> 4);
           if (leader && ok) {
 #pragma unroll
             for (int kk = 0; kk < kPairBlockK / 16; ++kk)
               mma_bf16_pair(d_tmem, a + 2 * kk, b + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+            if (kb + 1 < KB && kps > 1) {
+              const uint64_t a1 = a + (kPairHalfBytes >> 4);
+              const uint64_t b1 = b + static_cast<uint32_t>(rows_bytes >> 4);
+#pragma unroll
+              for (int kk = 0; kk < kPairBlockK / 16; ++kk)
+                mma_bf16_pair(d_tmem, a1 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+            }
             mma_commit_pair(&sm.empty[r.slot], 0x3);
           }
           __syncwarp();
