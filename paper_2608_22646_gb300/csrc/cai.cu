@@ -465,12 +465,13 @@ CommitParams commit_params(cai_ctx* c, int t, int64_t step_id) {
 
 // Multi-kernel step, kernel 1: the gather of this step's masked rows into
 // the compact operand (all rows at step zero).
-int launch_gather(cai_ctx* c, const void* hid, bool first, cudaStream_t stream,
+int launch_gather(cai_ctx* c, const void* hid, bool first, bool rows_ready, cudaStream_t stream,
                   const unsigned long long* stage_word = nullptr,
                   unsigned long long stage_seq = 0) {
   GatherParams gp{};
   gp.stage_word = stage_word;
   gp.stage_seq = stage_seq;
+  gp.prefetch = rows_ready ? 1 : 0;
   gp.hidden = static_cast<const __nv_bfloat16*>(hid);
   gp.hc = c->hc;
   gp.list = c->list;
@@ -635,7 +636,8 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
     const unsigned long long* word =
         stage_slot >= 0 && c->stage_by_word ? c->stage_seq_dev + stage_slot : nullptr;
     const int r =
-        launch_gather(c, hid, first, stream, word, static_cast<unsigned long long>(step_id + 1));
+        launch_gather(c, hid, first, stage_slot < 0, stream, word,
+                      static_cast<unsigned long long>(step_id + 1));
     if (r != CAI_OK) return r;
     if (stage_slot >= 0) {
       // stage2[stage_slot] may be refilled once the gather is done.
@@ -1328,7 +1330,8 @@ int cai_shard_head(cai_ctx* c, const void* hidden, void* triples, void* stream_v
   int r = multi_kernel_rows(c, hidden, stream, &hid);
   if (r != CAI_OK) return r;
   if (first) c->block_done_seen = false;
-  if ((r = launch_gather(c, hid, first, stream)) != CAI_OK) return r;
+  if ((r = launch_gather(c, hid, first, hid == hidden && is_device_ptr(hidden), stream)) != CAI_OK)
+    return r;
   if ((r = launch_pair_head(c, c->t_next, stream)) != CAI_OK) return r;
   ShardRowsParams sp{};
   sp.part = c->part;

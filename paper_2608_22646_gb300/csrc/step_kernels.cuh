@@ -39,12 +39,13 @@ struct GatherParams {
   float eps;
   const unsigned long long* stage_word;  // host rows staged by the side stream: read
   unsigned long long stage_seq;          // once *stage_word >= stage_seq (or null)
+  int prefetch;  // hidden is device memory that holds the rows already
 };
 
 __global__ void __launch_bounds__(kGatherThreads)
     gather_rows_kernel(const GatherParams p) {
   grid_launch_dependents();  // every thread: the CTA counts once all of them have
-  if (!p.first && !p.stage_word) {
+  if (!p.first && p.prefetch) {
     // While the previous step commits: the rows of its list, of which this
     // step's is a part, towards L2 (the weight has passed through it since).
     const int q = blockIdx.x * kGatherRowsPerCta + threadIdx.x / 64;
