@@ -214,7 +214,8 @@ int cai_config_default(cai_config* cfg, int32_t preset, int32_t B, int32_t P, in
 /*
  * Create a context.  W is the LM-head weight [V, H] bf16, row-major, host or
  * device memory.  It is read once, during this call, into the library's
- * packed copies (2 V H bytes each: one copy when B P <= 64, two otherwise);
+ * packed copy (2 V H bytes; two copies with CAI_PAIR_SWAP=0 in multi-kernel
+ * contexts);
  * the caller may free or change it afterwards.  All state starts at block 0,
  * t = 0, every token masked.  Allocates device memory and one page of mapped
  * pinned host memory.  Synchronous.

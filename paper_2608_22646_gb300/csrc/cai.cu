@@ -287,7 +287,7 @@ struct cai_ctx {
   // otherwise the step's stream waits for ev_copied.
   unsigned long long* stage_seq_dev = nullptr;
   bool stage_by_word = false;
-  bool fused = false;    // single-kernel step (B P <= 64)
+  bool fused = false;    // single-kernel step (fused_by_default)
   bool rows_head = false;  // the single-kernel step runs lm_head_rows_kernel
   int step_box = kBoxRowsB;  // rows per TMA box of a single-kernel step's rows: the rows-operand
                              // head loads a K block of them as one box (each copy costs its issue)
@@ -552,7 +552,7 @@ int multi_kernel_rows(cai_ctx* c, const void* hidden, cudaStream_t stream, const
   return CAI_OK;
 }
 
-// One denoising step.  Single-kernel step (B P <= 64): the LM-head kernel
+// One denoising step.  Single-kernel step: the LM-head kernel
 // reads the hidden states in place and its last CTA commits.  Otherwise:
 // gather -> LM head -> merge + commit.
 int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first);

@@ -59,8 +59,6 @@ namespace cai {
 
 constexpr int kRowsM = 128;                          // MMA M: rows of the step, padded
 constexpr int kRowsGroupRows = 256;                  // MMA N: vocabulary rows per group
-constexpr int kRowsWStage = kRowsGroupRows * 128;    // 32 KiB: one K block of the largest group
-constexpr int kRowsHStageMax = kRowsM * 128;         // 16 KiB: all 128 rows of a K block
 constexpr int kRowsTmemCols = 2 * kRowsGroupRows;    // two accumulators
 constexpr int kRowsEpiWarps = 8;                     // two per tensor-memory quarter
 constexpr int kRowsThreads = 64 + 32 * kRowsEpiWarps;
