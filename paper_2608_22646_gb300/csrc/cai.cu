@@ -820,7 +820,11 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   c->stats.pair_swap_max_n = c->swap_max_n;
   c->swap_on = c->swap_max_n > 0;
   if (c->swap_on && pair_swap_env() == 0) c->swap_max_n = pair_swap_width(cfg->H);
-  c->pair_kernel = c->norm ? lm_head_pair_kernel<true> : lm_head_pair_kernel<false>;
+  c->pair_kernel = pair_w_first(cfg->V, cfg->H, false) && c->BP <= 2 * kPairTileRows
+                       ? (c->norm ? lm_head_pair_kernel<true, false, true>
+                                  : lm_head_pair_kernel<false, false, true>)
+                       : (c->norm ? lm_head_pair_kernel<true, false, false>
+                                  : lm_head_pair_kernel<false, false, false>);
 
   // LM-head launch shape.  N chunk (positions per MMA), grid (one CTA per SM,
   // at least kMinCtaRows vocabulary rows per CTA), tile group size (tiles sharing one hidden

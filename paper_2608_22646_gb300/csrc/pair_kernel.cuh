@@ -195,6 +195,20 @@ __host__ __device__ inline int pair_tile_rows(int V, int n_pairs) {
   return V > 4 * 2 * kPairHalf * n_pairs ? kPairHalf : pair_even_rows(V, n_pairs);
 }
 
+// Whether W is read evict-first (kFirst, contexts of up to two row tiles).  A
+// weight well above what L2 keeps is better not kept: what stays is then an
+// unbroken part of it that the next step finds (1024 x 64000, M = 160: 35.9 ->
+// 32.7 us a step; 2048 x 50003 47.3 -> 43.6; 4096 x 126464 161.5 -> 158.2), a
+// smaller one is (1024 x 40000, 26.6 us, 27.2 evict-first).  Read in place from
+// row-major W the line lies higher: 1024 x 50003, 8 rows 17.4 us a call, 20.2
+// evict-first; 1024 x 64000 26.2, 24.7.  A template parameter: a branch between
+// the two forms in the producer's loop cost steps of two row tiles 4 %, a policy
+// operand with the normal priority small weights 5 % and steps of three row
+// tiles and more, which read W mostly from L2, 1.5 %.
+__host__ inline bool pair_w_first(int V, int H, bool in_place) {
+  return 2ll * V * H > (in_place ? 115ll : 95ll) << 20;
+}
+
 __host__ __device__ inline size_t pair_smem_bytes(int n_stages, bool swap) {
   return 1024 + static_cast<size_t>(n_stages) * kPairStageBytes + (swap ? kSwapXchBytes : 0) +
          static_cast<size_t>(2 * kPairMaxRing + 9) * 8 + 16 + 3 * kPairHalf * 4;
@@ -292,7 +306,7 @@ __device__ __forceinline__ void pair_drain(uint64_t* bar, uint32_t parity, uint3
 // kStatic: M_fixed rows that the caller passes, known at launch (M <= 256, W
 // row-major through the map's own swizzle); the set-up then comes before the
 // dependency wait.
-template <bool kNorm, bool kStatic = false>
+template <bool kNorm, bool kStatic, bool kFirst>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
     lm_head_pair_kernel(const __grid_constant__ CUtensorMap tm_a,
                         const __grid_constant__ CUtensorMap tm_w,
@@ -381,6 +395,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
   if (warp == 0) {
     // -------------------------------------------------------- producer --
     const uint64_t pol_a = policy_evict_last();
+    const uint64_t pol_w = policy_evict_first();
     const uint32_t full0 = mapa_shared(sm.full, 0);  // the even CTA's barriers
     const bool leader = elect_one();
     PairRing r;
@@ -399,6 +414,13 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
       // First row of this CTA's half of the tile's rows.
       const int a_row = j * rt_rows + static_cast<int>(rank) * (swap ? rt_rows / 2 : kPairHalf);
       const int w_row = (2 * v + static_cast<int>(rank)) * th;
+      auto load_w = [&](uint8_t* to, uint32_t bar, int kb) {  // K block kb of the W half
+        const int x = kb * p.w_dx, y = w_row * p.w_ry + kb * p.w_dy;
+        if constexpr (kFirst)
+          tma_load_2d_pair(to, tmw, bar, x, y, pol_w);
+        else
+          tma_load_2d_pair_nohint(to, tmw, bar, x, y);
+      };
       for (int kb = 0; kb < KB; kb += kps) {
         ok = ok && mbar_wait(&sm.empty[r.slot], r.phase ^ 1u, sm.abort, p.err, kErrWaitEmpty);
         if (leader && ok) {
@@ -412,18 +434,15 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
             // A: the W half; B: the CTA's rows, one box of box_rows.  (Two K
             // blocks: W, W, rows, rows.)
             uint8_t* rows = dst + kps * kPairHalfBytes;
-            tma_load_2d_pair_nohint(dst, tmw, bar, kb * p.w_dx, w_row * p.w_ry + kb * p.w_dy);
-            if (two)
-              tma_load_2d_pair_nohint(dst + kPairHalfBytes, tmw, bar, (kb + 1) * p.w_dx,
-                                      w_row * p.w_ry + (kb + 1) * p.w_dy);
+            load_w(dst, bar, kb);
+            if (two) load_w(dst + kPairHalfBytes, bar, kb + 1);
             tma_load_2d_pair(rows, &hm.box[q1], bar, kb * kPairBlockK, a_row, pol_a);
             if (two)
               tma_load_2d_pair(rows + rows_bytes, &hm.box[q1], bar, (kb + 1) * kPairBlockK, a_row,
                                pol_a);
           } else {
             tma_load_2d_pair(dst, &tm_a, bar, kb * kPairBlockK, a_row, pol_a);
-            tma_load_2d_pair_nohint(dst + kPairHalfBytes, tmw, bar, kb * p.w_dx,
-                                    w_row * p.w_ry + kb * p.w_dy);
+            load_w(dst + kPairHalfBytes, bar, kb);
           }
         }
         __syncwarp();

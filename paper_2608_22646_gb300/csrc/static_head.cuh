@@ -84,8 +84,9 @@ std::mutex g_setup_mutex;
 DeviceSetup g_setup[kStaticMaxDevices];
 EncodeFn g_encode = nullptr;
 
-void (*const static_kernel)(CUtensorMap, CUtensorMap, CUtensorMap, PairRowMaps,
-                            PairParams) = lm_head_pair_kernel<false, true>;
+// [1]: W read evict-first (pair_w_first).
+void (*const static_kernels[2])(CUtensorMap, CUtensorMap, CUtensorMap, PairRowMaps, PairParams) = {
+    lm_head_pair_kernel<false, true, false>, lm_head_pair_kernel<false, true, true>};
 
 // Once per device, with that device current: the device addresses of the
 // static scratch (a host-side name of a __device__ array is not a device
@@ -110,7 +111,7 @@ int setup_device(int dev, DeviceSetup** out) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
             cudaSuccess ||
-        cudaFuncGetAttributes(&attr, static_kernel) != cudaSuccess) {
+        cudaFuncGetAttributes(&attr, static_kernels[0]) != cudaSuccess) {
       cudaGetLastError();
       return CAI_ERR_CUDA;
     }
@@ -123,9 +124,11 @@ int setup_device(int dev, DeviceSetup** out) {
     qc.gridDim = dim3(static_cast<unsigned>(sms & ~1));
     qc.blockDim = dim3(kPairThreads);
     qc.dynamicSmemBytes = d.smem;
-    if (cudaFuncSetAttribute(static_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(static_kernels[0], cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(d.smem)) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&d.pairs, static_kernel, &qc) != cudaSuccess ||
+        cudaFuncSetAttribute(static_kernels[1], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(d.smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&d.pairs, static_kernels[0], &qc) != cudaSuccess ||
         d.pairs < 1) {
       cudaGetLastError();
       return CAI_ERR_CUDA;
@@ -216,8 +219,8 @@ extern "C" int cai_head_rows_static(const void* W, int32_t V, int32_t H, const v
   // An error left pending by earlier, unrelated work is not this call's.
   cudaGetLastError();
   // If the LM head did not launch, the merge would read a previous call's partials.
-  if (launch_pdl(true, static_kernel, 2 * pairs, kPairThreads, d->smem, s, tm_r, tm_w, tm_w, maps,
-                 pp) != cudaSuccess) {
+  if (launch_pdl(true, static_kernels[pair_w_first(V, H, true) ? 1 : 0], 2 * pairs, kPairThreads,
+                 d->smem, s, tm_r, tm_w, tm_w, maps, pp) != cudaSuccess) {
     cudaGetLastError();
     return CAI_ERR_CUDA;
   }
