@@ -197,6 +197,21 @@ cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), int grid, int block, 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// The most dynamic shared memory a launch of `kernel` may ask for on this
+// device (the opt-in size less the kernel's static shared memory), also set as
+// the kernel's launch limit.  That limit belongs to the function on the device,
+// not to a context: set to one context's own size, a context made later with a
+// smaller one would make the steps of a live context fail to launch.  Every
+// context and thread sets the same value.
+template <typename K>
+bool open_dynamic_smem(K* kernel, int smem_optin, size_t* limit) {
+  cudaFuncAttributes a{};
+  if (cudaFuncGetAttributes(&a, kernel) != cudaSuccess) return false;
+  *limit = static_cast<size_t>(smem_optin) - a.sharedSizeBytes;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(*limit)) == cudaSuccess;
+}
+
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -882,14 +897,12 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     const int per = c->gmax > 1 ? (tight ? c->gmax : c->gmax - 1) : 1;
     return c->gmax == 1 ? stages : (stages + per - 1) / per + 1;
   };
-  // Dynamic shared memory may use what the kernel's static shared memory leaves.
-  cudaFuncAttributes head_attr{};
-  if (cudaFuncGetAttributes(&head_attr, c->head_kernel) != cudaSuccess) {
+  size_t dyn_limit = 0;
+  if (!open_dynamic_smem(c->head_kernel, smem_optin, &dyn_limit)) {
     cudaGetLastError();
     delete c;
     return CAI_ERR_CUDA;
   }
-  const size_t dyn_limit = static_cast<size_t>(smem_optin) - head_attr.sharedSizeBytes;
   const int scap = env_int("CAI_HEAD_STAGES");
   int stages = scap >= 2 && scap <= 16 ? scap : 12;
   while (stages > 2 && head_smem_bytes(stages, bslots_for(stages), c->b_slot_bytes,
@@ -907,13 +920,12 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     c->rows_head = true;
     c->step_box = c->rows_cap;
     c->head_kernel = c->norm ? lm_head_rows_kernel<true> : lm_head_rows_kernel<false>;
-    cudaFuncAttributes ra{};
-    if (cudaFuncGetAttributes(&ra, c->head_kernel) != cudaSuccess) {
+    size_t rlimit = 0;
+    if (!open_dynamic_smem(c->head_kernel, smem_optin, &rlimit)) {
       cudaGetLastError();
       delete c;
       return CAI_ERR_CUDA;
     }
-    const size_t rlimit = static_cast<size_t>(smem_optin) - ra.sharedSizeBytes;
     // kRowsInFlight bytes of W in stages of the largest group's size;
     // CAI_ROWS_STAGES sets the ring's depth (tuning knob).
     int most = 0;
@@ -945,13 +957,12 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   // can be resident at once.
   if (c->use_pair) {
     c->n_vt = (cfg->V + kPairTileVocab - 1) / kPairTileVocab;
-    cudaFuncAttributes pa{};
-    if (cudaFuncGetAttributes(&pa, c->pair_kernel) != cudaSuccess) {
+    size_t plimit = 0;
+    if (!open_dynamic_smem(c->pair_kernel, smem_optin, &plimit)) {
       cudaGetLastError();
       delete c;
       return CAI_ERR_CUDA;
     }
-    const size_t plimit = static_cast<size_t>(smem_optin) - pa.sharedSizeBytes;
     // CAI_PAIR_STAGES caps the ring depth (tuning knob; results do not depend on it).
     const int pcap = env_int("CAI_PAIR_STAGES");
     int ps = pcap >= 2 && pcap < 6 ? pcap : 6;
@@ -961,12 +972,6 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     const int rmax = env_int("CAI_PAIR_RING_MAX");
     if (rmax >= 2 && rmax <= kPairMaxRing) c->pair_ring_max = rmax;
     int clusters = 0;
-    if (cudaFuncSetAttribute(c->pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(c->pair_smem)) != cudaSuccess) {
-      cudaGetLastError();
-      delete c;
-      return CAI_ERR_CUDA;
-    }
     cudaLaunchConfig_t qc = {};
     qc.gridDim = dim3(static_cast<unsigned>(sms & ~1));
     qc.blockDim = dim3(kPairThreads);
@@ -1185,9 +1190,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   // small gather and merge CTAs can be resident on an SM beside an LM-head
   // CTA; under programmatic dependent launch they then start, and wait, while
   // the neighbouring kernel still runs.
-  if (cudaFuncSetAttribute(c->head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(c->head_smem)) != cudaSuccess ||
-      cudaFuncSetAttribute(c->head_kernel,
+  if (cudaFuncSetAttribute(c->head_kernel,
                            cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
       cudaFuncSetAttribute(gather_rows_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
