@@ -365,13 +365,14 @@ int validate(const cai_config* c) {
 constexpr size_t kGuardBytes = 256;
 constexpr unsigned char kGuardByte = 0xC3;
 
-int alloc_into(cai_ctx* c, void** dst, size_t bytes) {
+int alloc_into(cai_ctx* c, void** dst, size_t bytes, cudaStream_t stream) {
   const size_t padded = (bytes + 255) / 256 * 256;
   int r = dev_alloc(dst, padded + kGuardBytes);
   if (r != CAI_OK) return r;
   c->allocs.push_back(*dst);
   c->alloc_bytes.push_back(padded);
-  if (cudaMemset(static_cast<char*>(*dst) + padded, kGuardByte, kGuardBytes) != cudaSuccess)
+  if (cudaMemsetAsync(static_cast<char*>(*dst) + padded, kGuardByte, kGuardBytes, stream) !=
+      cudaSuccess)
     return CAI_ERR_CUDA;
   return CAI_OK;
 }
@@ -1000,12 +1001,16 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   const size_t BL = static_cast<size_t>(cfg->B) * c->L;
   const size_t BN = static_cast<size_t>(cfg->B) * cfg->n_blocks;
   void* p;
-#define CAI_ALLOC(field, type, count)                                  \
-  if ((r = alloc_into(c, &p, sizeof(type) * (count))) != CAI_OK) {    \
-    release(c);                                                        \
-    delete c;                                                          \
-    return r;                                                          \
-  }                                                                    \
+  // Buffers are cleared and filled on the caller's stream, which is waited for at
+  // the end: a memset or copy on the legacy default stream is ordered before
+  // nothing that a non-blocking stream runs.
+  const cudaStream_t init_stream = static_cast<cudaStream_t>(stream);
+#define CAI_ALLOC(field, type, count)                                            \
+  if ((r = alloc_into(c, &p, sizeof(type) * (count), init_stream)) != CAI_OK) { \
+    release(c);                                                                  \
+    delete c;                                                                    \
+    return r;                                                                    \
+  }                                                                              \
   field = static_cast<type*>(p);
   CAI_ALLOC(c->st.tok, int, BL)
   CAI_ALLOC(c->st.conf, float, BL)
@@ -1026,7 +1031,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     CAI_ALLOC(c->h_prev, __nv_bfloat16, static_cast<size_t>(c->BP) * cfg->H)
     CAI_ALLOC(c->drift_ratio, float, c->BP)
     CAI_ALLOC(c->drift_count, unsigned, cfg->B)
-    if (cudaMemset(c->drift_count, 0, sizeof(unsigned) * cfg->B) != cudaSuccess) {
+    if (cudaMemsetAsync(c->drift_count, 0, sizeof(unsigned) * cfg->B, init_stream) !=
+        cudaSuccess) {
       release(c);
       delete c;
       return CAI_ERR_CUDA;
@@ -1036,7 +1042,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   CAI_ALLOC(c->row_of, int, c->BP)
   CAI_ALLOC(c->d_M, int, 1)
   CAI_ALLOC(c->ticket, unsigned, 2)
-  if (cudaMemset(c->ticket, 0, 8) != cudaSuccess) {  // every step leaves it at zero
+  if (cudaMemsetAsync(c->ticket, 0, 8, init_stream) != cudaSuccess) {  // every step leaves it at zero
     release(c);
     delete c;
     return CAI_ERR_CUDA;
@@ -1065,7 +1071,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
     c->stage2[0] = c->hidden_stage;
     CAI_ALLOC(c->stage2[1], uint8_t, static_cast<size_t>(c->BP) * cfg->H * 2)
     CAI_ALLOC(c->stage_seq_dev, unsigned long long, 2)
-    if (cudaMemset(c->stage_seq_dev, 0, 16) != cudaSuccess) {
+    if (cudaMemsetAsync(c->stage_seq_dev, 0, 16, init_stream) != cudaSuccess) {
       release(c);
       delete c;
       return CAI_ERR_CUDA;
@@ -1078,7 +1084,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   if (c->head_in_step) CAI_ALLOC(c->wpk, uint8_t, static_cast<size_t>(units) * kUnitRows * 2 * cfg->H)
   if (c->norm) {
     CAI_ALLOC(c->inv_r, float, c->rows_cap)
-    if (cudaMemset(c->inv_r, 0, sizeof(float) * c->rows_cap) != cudaSuccess) {
+    if (cudaMemsetAsync(c->inv_r, 0, sizeof(float) * c->rows_cap, init_stream) != cudaSuccess) {
       release(c);
       delete c;
       return CAI_ERR_CUDA;
@@ -1093,8 +1099,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
       delete c;
       return r;
     }
-    if (cudaMemcpy(g_tmp, g, static_cast<size_t>(cfg->H) * 2, cudaMemcpyHostToDevice) !=
-        cudaSuccess) {
+    if (cudaMemcpyAsync(g_tmp, g, static_cast<size_t>(cfg->H) * 2, cudaMemcpyHostToDevice,
+                        init_stream) != cudaSuccess) {
       cudaFree(g_tmp);
       release(c);
       delete c;
@@ -1111,8 +1117,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
       delete c;
       return r;
     }
-    if (cudaMemcpy(w_tmp, W, static_cast<size_t>(cfg->V) * cfg->H * 2, cudaMemcpyHostToDevice) !=
-        cudaSuccess) {
+    if (cudaMemcpyAsync(w_tmp, W, static_cast<size_t>(cfg->V) * cfg->H * 2, cudaMemcpyHostToDevice,
+                        init_stream) != cudaSuccess) {
       cudaFree(w_tmp);
       if (g_tmp) cudaFree(g_tmp);
       release(c);
@@ -1124,22 +1130,22 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   {
     const int pack_grid = 8 * sms;
     if (c->rows_head)
-      pack_weight_rows_kernel<<<pack_grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      pack_weight_rows_kernel<<<pack_grid, 256, 0, init_stream>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wpk), cfg->V, cfg->H, units,
           c->G, g_dev);
     else if (c->head_in_step)
-      pack_weight_kernel<<<pack_grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      pack_weight_kernel<<<pack_grid, 256, 0, init_stream>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wpk), cfg->V, cfg->H, units,
           c->G, c->gmax, g_dev);
     if (c->use_pair)
-      pack_w_tiles_kernel<<<pack_grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      pack_w_tiles_kernel<<<pack_grid, 256, 0, init_stream>>>(
           static_cast<const uint4*>(w_src), static_cast<uint4*>(c->wt), cfg->V, cfg->H,
           pair_w_run(cfg->V, c->pair_th1),
           static_cast<int>(pair_w_rows(cfg->V, cfg->H, pair_w_run(cfg->V, c->pair_th1)) /
                            (cfg->H / kPairBlockK) / kUnitRows),
           g_dev);
     const cudaError_t e1 = cudaGetLastError();
-    const cudaError_t e2 = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
+    const cudaError_t e2 = cudaStreamSynchronize(init_stream);
     if (w_tmp) cudaFree(w_tmp);
     if (g_tmp) cudaFree(g_tmp);
     if (e1 != cudaSuccess || e2 != cudaSuccess) {
@@ -1213,6 +1219,8 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
                : 2 + (c->head_in_step ? 1 : 0) + (c->use_pair ? 1 : 0) + (c->need_reduce ? 1 : 0) +
                      (c->shard ? 2 : 0);
   r = cai_reset(c, stream);
+  // The first step may come on any stream.
+  if (r == CAI_OK && cudaStreamSynchronize(init_stream) != cudaSuccess) r = CAI_ERR_CUDA;
   if (r != CAI_OK) {
     release(c);
     delete c;

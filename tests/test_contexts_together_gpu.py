@@ -79,3 +79,35 @@ def test_both_full_size_models(names):
     finally:
         for ctx, _, _ in made:
             cai.cai_free(ctx)
+
+
+@pytest.mark.parametrize("B,flags", [(2, 0), (5, 0), (5, cai.CAI_DIAGNOSTICS)])
+@pytest.mark.parametrize("host", [False, True])
+def test_init_on_a_side_stream(B, flags, host):
+    # A context made on one non-blocking stream while the default stream is
+    # busy (its work is ordered before nothing of theirs), stepped on another
+    # as soon as cai_init has returned: the states of a context made and
+    # stepped on the default stream.
+    P, H, V, T = 40, 256, 3000, 4
+    wl = synth.Workload("side", B=B, H=H, V=V, gen_len=P, P=P, T=T, a0="u04")
+    W = synth.lm_head_weight(V, H, seed=3, device="cuda")
+    hidden = [synth.HiddenStates(wl, W, "calibrated", seed=4)(0, t) for t in range(T)]
+    g = synth.final_norm_weight(H, seed=9, device="cuda")
+    cfg = cai.cai_config_default(cai.CAI_PRESET_LLADA, B, P, H, V, T, 1)
+    cfg.flags |= flags
+    ends = []
+    for side in (False, True):
+        torch.cuda.synchronize()
+        made, run = (torch.cuda.Stream(), torch.cuda.Stream()) if side else (None, None)
+        if side:
+            torch.cuda._sleep(400_000_000)
+        ctx = cai.cai_init_rmsnorm(cfg, W.cpu() if host else W, g.cpu() if host else g, 1e-5, made)
+        try:
+            for t in range(T):
+                (cai.cai_denoise_step if t else cai.cai_first_step)(ctx, hidden[t], run)
+            ends.append(cai.cai_state_download(ctx))
+            assert cai.cai_test_check_guards(ctx) == 0
+        finally:
+            cai.cai_free(ctx)
+    for f in ends[0]:
+        assert np.array_equal(ends[0][f], ends[1][f], equal_nan=f == "drift"), f
