@@ -393,7 +393,10 @@ void cai_free(cai_ctx* ctx);
  * For each of the M rows of `rows` ([M, H] bf16, device), computes
  * conf[i] = max_v softmax(W rows[i])_v and argmax[i] = the lowest v reaching
  * that maximum, against the caller's W ([V, H] bf16 row-major, device, read in
- * place).  conf (float) and argmax (int32) are device arrays of M entries.
+ * place).  A row without a softmax (a NaN or +inf logit, or none above -inf)
+ * gets the confidence NaN and still an index below V; so do the steps of a
+ * context on the default kernels, which never commit such a row by its
+ * confidence.  conf (float) and argmax (int32) are device arrays of M entries.
  * Asynchronous on `stream`.  Limits: 1 <= M <= 256, V >= 128, H % 64 == 0 and
  * 64 <= H <= 16384 (else CAI_ERR_SHAPE); W and rows 16-byte aligned, and all
  * four pointers device (or managed) memory of the current device (else

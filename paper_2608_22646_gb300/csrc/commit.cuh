@@ -241,7 +241,7 @@ __device__ void merge_rows(const CommitParams& p, int b0, int nb, CommitSmem& cs
       int ix;
       warp_merge(q[j], m, s, ix);
       const int i = base + j * nwarps;
-      const float c = 1.0f / s;  // max_v p_v = exp(m - LSE) = 1 / sum_v exp(z_v - m)
+      const float c = row_confidence(m, s, ix);
       if (lane == 0) {
         if (kAll) {
           cs.conf[i] = c;

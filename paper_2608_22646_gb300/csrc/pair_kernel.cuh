@@ -542,7 +542,7 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
         for (int k = 0; k < 4 * kSwapChunks; ++k) {
           am[k] = kNegBig;
           as[k] = 0.0f;
-          aix[k] = nrow > 0 ? vrow : INT_MAX;
+          aix[k] = INT_MAX;
         }
       }
       if (!mbar_wait(&sm.accf[acc], (i >> 1) & 1, sm.abort, p.err, kErrWaitAccFull)) break;
@@ -613,8 +613,6 @@ __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kPairRegs)
           const float4 a = sm.xch[(buf * 4 + w) * kPairTileVocab + et];
           merge_tri(m, sum, ix, a.x, a.y, __float_as_int(a.z));
         }
-        // Valid rows but no logit above the empty maximum (all -inf): no softmax.
-        if (m == kNegBig && ix != INT_MAX) sum = __int_as_float(0x7fc00000);
         const size_t row = static_cast<size_t>(row0 + et);
         if (per_row > 0)
           p.part[row * per_row + 2 * (pair / n_rt) + static_cast<int>(rank)] =

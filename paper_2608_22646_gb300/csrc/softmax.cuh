@@ -105,6 +105,17 @@ __device__ __forceinline__ void warp_merge(const float4 (&q)[kN], float& m, floa
   ix = __reduce_min_sync(0xffffffffu, ix);
 }
 
+// A row's confidence max_v p_v = exp(m - LSE) = 1 / S from its merged triple.  A
+// row without a logit above the empty maximum (all NaN or -inf) has no softmax:
+// its confidence is NaN, which passes no threshold, and its index 0, the lowest
+// of the equal ones, so that what is stored as an argmax always is one.  (A +inf
+// logit makes S, and so the confidence, NaN by itself: exp2(inf - inf).)
+__device__ __forceinline__ float row_confidence(float m, float s, int& ix) {
+  if (m > kNegBig) return 1.0f / s;
+  ix = 0;
+  return __int_as_float(0x7fc00000);
+}
+
 // 32 lanes x 32 columns of online-softmax triples -> lane l holds the merge of
 // column l over the 32 lanes, in m[0], s[0], ix[0].  Five halving steps: at
 // width w each lane keeps half of its live columns and receives the partner's

@@ -57,7 +57,8 @@ __global__ void merge_rows_static_kernel(const float4* part, uint32_t* err, int 
     warp_merge(q, m, s, ix);
   }
   if (lane == 0 && row < M) {
-    conf[row] = bad ? __int_as_float(0x7fc00000) : 1.0f / s;
+    const float c = row_confidence(m, s, ix);
+    conf[row] = bad ? __int_as_float(0x7fc00000) : c;
     argmax[row] = bad ? -1 : ix;
   }
   __syncthreads();  // every warp of this CTA has read the error word
