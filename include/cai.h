@@ -24,14 +24,18 @@
  * before it in the stream still runs, and waits for that kernel to complete
  * before touching anything it produces (setting CAI_PDL=0 in the environment
  * before cai_init launches them plainly instead).  With B P <= 64, or B P <= 128
- * and a weight of 8 MiB or more, a step is one kernel: the LM head over every row of the block, whose last CTA applies
- * the commit rule; it streams W before the previous step has committed and
- * waits for it only to write its partials and to commit (CAI_FUSED_MAX_BP=n
- * moves the limit, up to 256).  That LM head puts the rows in the MMA's A
- * operand and 256 vocabulary rows in N (up to 128 rows; CAI_ROWS_HEAD=0 uses
- * the swapped-operand kernel instead, W in A and the rows in N).  Otherwise a step is gather, LM head,
- * merge + commit.  The LM head is the CTA-pair
- * kernel (tcgen05 cta_group::2), which picks its orientation per step from
+ * and a weight of 8 MiB or more, a step is one kernel: the LM head over every
+ * row of the block, whose last CTA applies the commit rule; it streams W before
+ * the previous step has committed and waits for it only to write its partials
+ * and to commit (CAI_FUSED_MAX_BP=n moves the limit, up to 256).  One thing such
+ * a step reads without waiting: with B P <= 64, the caller's device rows.  A
+ * kernel that writes them directly before the step must not start its
+ * dependents early (griddepcontrol.launch_dependents before its last write;
+ * kernels that never execute it are fine), or CAI_PDL=0 has to be set.  That
+ * LM head puts the rows in the MMA's A operand and 256 vocabulary rows in N (up
+ * to 128 rows; CAI_ROWS_HEAD=0 uses the swapped-operand kernel instead, W in A
+ * and the rows in N).  Otherwise a step is gather, LM head, merge + commit.  The
+ * LM head is the CTA-pair kernel (tcgen05 cta_group::2), which picks its orientation per step from
  * the masked-row count M: the rows as MMA N in row tiles of equal width (a
  * multiple of 32) while that width is at most a limit that grows with H (224
  * from H = 3072 on), else as MMA M in 256-row tiles.  A kernel that merges each row's per-tile partials follows it only

@@ -33,15 +33,17 @@ std::atomic<int> g_head_grid_limit{0};
 // Whether a context of `rows` = B P positions runs single-kernel steps by
 // default.  They decode every row of the block each step and save the gather,
 // the commit kernel and three kernel boundaries; the rows-operand LM head pads
-// the rows to 128 anyway, and the next step's weight stream runs under the
-// commit.  Measured, microseconds a step back to back, single- against
-// multi-kernel with every row masked (multi-kernel at 8 rows in brackets):
-// 96 rows, 4096 x 126464 134 against 159 (152), 1024 x 50003 18.4 against 28.2
-// (21); 128 rows, 142 against 161, 3584 x 152064 145 against 165, 1024 x 22000
-// 11.7 against 21.6 (15); alone 165.8 against 174 at 96 rows and 174.6 against
-// 174.6 at 128.  With a weight of a few MB both are short chains of latencies
-// that differ little, and above 64 rows the multi-kernel step stays: it gets
-// shorter as rows commit.
+// the rows to 128 anyway.  Above 64 rows a step waits for the kernel before it
+// in the stream before it reads device rows, as a multi-kernel step does (its
+// producer may start its dependents early); only the first stages of the weight
+// stream ahead of that.  Measured, microseconds for a whole block of 8 to 12
+// steps, back to back, single- against multi-kernel: 96 rows, 4096 x 126464
+// 1224 against 1264, 1024 x 4096 152 against 178; 99 rows, 1024 x 50003 255
+// against 271, 256 x 16384 193 against 215; 128 rows, 4096 x 126464 1242 against
+// 1271, 3584 x 152064 1297 against 1306, 2048 x 50003 391 against 394, 1024 x
+// 22000 183 against 190.  With a weight of a few MB both are short chains of
+// latencies that differ little, and above 64 rows the multi-kernel step stays:
+// it gets shorter as rows commit.
 constexpr int kFusedMaxRows = 64;       // any weight
 constexpr int kFusedMaxRowsLarge = 128; // weights of at least ...
 constexpr long long kFusedLargeBytes = 8ll << 20;
@@ -683,6 +685,9 @@ int step_impl(cai_ctx* c, const void* hidden, void* stream_v, bool first) {
     hp.stage_seq = static_cast<unsigned long long>(step_id + 1);
   }
   hp.prefetch = c->use_pair ? 0 : 1;
+  // (see fused_by_default; staged rows have a wait of their own, and up to 64
+  // rows the header asks for a producer that does not start dependents early)
+  hp.wait_rows = c->fused && c->BP > kFusedMaxRows && stage_slot < 0 ? 1 : 0;
   hp.first = first ? 1 : 0;
   hp.part = c->part;  // (single-kernel step: cp.part, below)
   hp.err = c->err;

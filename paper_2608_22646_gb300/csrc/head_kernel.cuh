@@ -81,6 +81,7 @@ struct HeadParams {
   const unsigned long long* stage_word;  // single-kernel step on staged host rows: the rows
   unsigned long long stage_seq;          // are read once *stage_word >= stage_seq (or null)
   int prefetch;        // stream the first W stages before the dependency wait
+  int wait_rows;       // single-kernel step: wait for the kernel before it to read the rows
   int first;           // the step is a block's step zero (every position masked)
   float4* part;        // [rows_cap, G] partial (m2, S, idx bits, 0) per CTA
   uint32_t* err;       // error word
@@ -428,7 +429,8 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
   // that does (the masked-row count, the gathered rows, the partial buffer,
   // the commit state) is touched only after grid_dependency_wait().  A
   // single-kernel step reads nothing the previous step writes before its
-  // partials, so only its epilogue and its commit wait.
+  // partials, so only its epilogue and its commit wait (and, with wait_rows,
+  // whoever reads the caller's rows).
   // When most steps go to the pair kernel, copies started before M is known
   // would mostly be wasted, so the launch asks for none.
   const int n_pre = p.prefetch ? min(p.n_stages, pl.n_tiles * KB) : 0;
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
                         p.wpk + pl.stage_offset(g, kb, t, p.H), bytes, &sm.full_a[i], pol_w);
             }
       }
-      if (!p.fused) grid_dependency_wait();
+      if (!p.fused || p.wait_rows) grid_dependency_wait();
       const int M = rows_to_decode(p.d_M, p.fused, p.M_fixed, p.max_M);
       const int n_chunks = (M + kChunkN - 1) / kChunkN;
       Ring ra, rb;
@@ -615,6 +617,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
     if constexpr (kNorm) {
       __shared__ float s_scale[kChunkN];
       if (p.fused) {
+        if (p.wait_rows) grid_dependency_wait();
         epilogue_row_scales<4>(p.hid, M, p.H, p.norm_eps, s_scale, ew, lane);
         scale = s_scale;
       }

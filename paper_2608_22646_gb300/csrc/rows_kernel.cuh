@@ -249,6 +249,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     Ring r;
     int issued = 0;
     bool ok = true, decided = !spec;
+    if (p.wait_rows) grid_dependency_wait();
     // Rows copied from the host on the context's side stream: wait (bounded)
     // for that copy's sequence word before the first row load.
     if (leader && p.stage_word &&
@@ -382,6 +383,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
       // group accumulates.  Nothing here depends on an earlier kernel, so the
       // accumulators are drained as in a step without the norm.
       __shared__ float s_scale[kRowsM];
+      if (p.wait_rows) grid_dependency_wait();
       epilogue_row_scales<kRowsEpiWarps>(p.hid, M, p.H, p.norm_eps, s_scale, warp - 2, lane);
       if (row < M) rs = kLog2e * s_scale[row];
     }
