@@ -298,8 +298,9 @@ def _roofline(wl, st0, stats1, head_ms, head_launches, step_ms, ms, steps, steps
     elif kps == 1:
         kernel = "lm_head_softmax_kernel (single-kernel step: LM head, softmax and commit)"
     elif stats1["pair_swap_max_n"] >= 32:
-        kernel = (f"lm_head_pair_kernel (every step; swapped orientation for tiles up to "
-                  f"{stats1['pair_swap_max_n']} rows wide)")
+        limit = stats1["pair_swap_limit"]
+        kernel = ("lm_head_pair_kernel (every step; " + (
+            f"swapped orientation for tiles up to {limit} rows wide)" if limit else "unswapped)"))
     elif stats1["pair_grid"]:
         kernel = "lm_head_pair_kernel (>= 32 rows) / lm_head_softmax_kernel (< 32 rows)"
     else:
@@ -385,7 +386,7 @@ def measure(cai, wl, generator, args, dist, dev, steps, warmup, with_e2e=True, c
         if dist:
             dist.barrier()
     ms = ev0.elapsed_time(ev1)
-    stats1 = cai.cai_get_stats(ctx)
+    stats1 = dict(cai.cai_get_stats(ctx), pair_swap_limit=cai.cai_pair_swap_limit(ctx))
     st1 = cai.cai_state_download(ctx)
     assert np.array_equal(st1["m_hist"], st0["m_hist"]), "trajectory changed between runs"
     gpu_launches = stats1["launches"] - stats0["launches"]

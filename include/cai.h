@@ -199,12 +199,9 @@ typedef struct cai_stats {
                                LM head(s), row merge if needed, commit (2 to 5)    */
   double step_ms;           /* summed device time of profiled steps, every kernel  */
   int32_t pair_grid;        /* CTAs of the CTA-pair LM head (0: not used)          */
-  int32_t pair_swap_max_n;  /* steps whose tile width in the swapped orientation
-                               (masked rows in the MMA N dimension) is at most
-                               this may run swapped on the pair LM head (0: never);
-                               unless CAI_PAIR_SWAP_MAX_N is set, the limit in use
-                               follows H: 0 below 384, 64 below 768, 96 below 1536,
-                               192 below 3072, then 224                            */
+  int32_t pair_swap_max_n;  /* the setting of the widest swapped tile: CAI_PAIR_SWAP_MAX_N,
+                               192 when it is not set, 0 when swapped steps are turned
+                               off; cai_pair_swap_limit tells the limit in use     */
   int32_t pair_stages;      /* pipeline stages of the pair LM head                 */
   int32_t head_rows;        /* 1: single-kernel steps run the LM head with the rows
                                as the MMA's A operand (B P <= 128), 0: otherwise   */
@@ -365,6 +362,14 @@ int cai_read_tokens(cai_ctx* ctx, int32_t* host_tokens, void* stream);
  * cai_get_stats synchronises the events and reports the sums. */
 int cai_profile(cai_ctx* ctx, int32_t enable);
 int cai_get_stats(cai_ctx* ctx, cai_stats* out);
+
+/* The limit in use in the context's multi-kernel steps: a step runs swapped on
+ * the pair LM head (masked rows in the MMA N dimension) when its tiles are then
+ * at most *limit rows wide (0: never).  CAI_PAIR_SWAP_MAX_N where it was set at
+ * cai_init, else by H: 0 below 384, 64 below 768, 96 below 1536, 192 below 3072,
+ * 224 from there; 0 in contexts that do not use the pair LM head or have
+ * CAI_PAIR_SWAP=0.  Host only.  Errors: CAI_ERR_ARG. */
+int cai_pair_swap_limit(const cai_ctx* ctx, int32_t* limit);
 
 /* The context's device error word, which kernels set when a bounded wait
  * gives up (the reason behind CAI_ERR_DEVICE): one bit per kind of wait,

@@ -56,7 +56,7 @@ EXPORTS = ("cai_config_default", "cai_init", "cai_init_rmsnorm", "cai_first_step
            "cai_test_check_guards",
            "cai_head_rows_static", "cai_test_static_wait_timeout",
            "cai_init_vocab_shard", "cai_shard_rows", "cai_shard_head", "cai_shard_commit",
-           "cai_device_error_bits")
+           "cai_device_error_bits", "cai_pair_swap_limit")
 
 
 class CaiError(RuntimeError):
@@ -121,6 +121,7 @@ def _load():
         "cai_read_tokens": (ctypes.c_int, [vp, vp, vp]),
         "cai_profile": (ctypes.c_int, [vp, i32]),
         "cai_get_stats": (ctypes.c_int, [vp, ctypes.POINTER(cai_stats)]),
+        "cai_pair_swap_limit": (ctypes.c_int, [vp, ctypes.POINTER(i32)]),
         "cai_device_error_bits": (ctypes.c_int, [vp, ctypes.POINTER(ctypes.c_uint32)]),
         "cai_free": (None, [vp]),
         "cai_strerror": (ctypes.c_char_p, [ctypes.c_int]),
@@ -395,6 +396,13 @@ def cai_get_stats(ctx: Ctx) -> dict:
     s = cai_stats()
     _check(lib().cai_get_stats(ctx.handle, ctypes.byref(s)), "cai_get_stats")
     return {n: getattr(s, n) for n, _ in cai_stats._fields_}
+
+
+def cai_pair_swap_limit(ctx: Ctx) -> int:
+    """Widest tile that the context's multi-kernel steps run swapped (0: never)."""
+    n = ctypes.c_int32(0)
+    _check(lib().cai_pair_swap_limit(ctx.handle, ctypes.byref(n)), "cai_pair_swap_limit")
+    return n.value
 
 
 DEVERR_NAMES = ("wait_empty", "wait_full", "wait_acc_full", "wait_acc_empty", "drain", "bad_row",

@@ -78,9 +78,10 @@ int pair_swap_env() {
   return v >= 32 && v <= 256 ? v : 0;
 }
 
-// Widest tile the pair kernel runs in the swapped orientation (masked rows in
-// the MMA N dimension, 32-row granularity): CAI_PAIR_SWAP_MAX_N (32..256), or
-// 0 with CAI_PAIR_SWAP=0; default 192.
+// The setting of the widest tile the pair kernel runs in the swapped
+// orientation (masked rows in the MMA N dimension, 32-row granularity):
+// CAI_PAIR_SWAP_MAX_N (32..256), or 0 with CAI_PAIR_SWAP=0.  192 stands for "not
+// set": the limit in use is then pair_swap_width(H).
 int pair_swap_max_n() {
   const char* e = std::getenv("CAI_PAIR_SWAP");
   if (e && e[0] == '0') return 0;
@@ -838,7 +839,7 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
   c->use_pair = shard || (!c->fused && pair_enabled());
   c->swap_max_n = c->use_pair ? pair_swap_max_n() : 0;
   if (shard && c->swap_max_n < kSwapColStep) c->swap_max_n = 192;
-  c->stats.pair_swap_max_n = c->swap_max_n;
+  c->stats.pair_swap_max_n = c->swap_max_n;  // the setting; the limit by H follows
   c->swap_on = c->swap_max_n > 0;
   if (c->swap_on && pair_swap_env() == 0) c->swap_max_n = pair_swap_width(cfg->H);
   c->pair_kernel = pair_w_first(cfg->V, cfg->H, false) && c->BP <= 2 * kPairTileRows
@@ -1588,6 +1589,12 @@ int cai_get_stats(cai_ctx* c, cai_stats* out) {
   c->stats.head_profiled += static_cast<int64_t>(c->ev_used / 4);
   c->ev_used = 0;
   *out = c->stats;
+  return CAI_OK;
+}
+
+int cai_pair_swap_limit(const cai_ctx* c, int32_t* limit) {
+  if (!c || !limit) return CAI_ERR_ARG;
+  *limit = c->swap_max_n;
   return CAI_OK;
 }
 
