@@ -194,7 +194,8 @@ def _buf(x, what: str, dtype: str) -> int | None:
     dt = x.dtype
     name = _DTYPE_NAMES.get(dt)
     if name is None:
-        name = _DTYPE_NAMES[dt] = str(dt).removeprefix("torch.")
+        full = str(dt)  # "torch.bfloat16"; another library's dtype has no name here
+        name = _DTYPE_NAMES[dt] = full[6:] if full.startswith("torch.") else ""
     if name != dtype or not x.is_contiguous():
         raise ValueError(f"{what}: expected a contiguous torch.{dtype} tensor "
                          f"(got {x.dtype}, contiguous={x.is_contiguous()})")
