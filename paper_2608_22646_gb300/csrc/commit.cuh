@@ -138,7 +138,7 @@ __device__ __forceinline__ void commit_load(const CommitParams& p, int b0, int n
     const int q = i / p.P;
     const size_t g = static_cast<size_t>(b0 + q) * p.L + p.blk * p.P + (i - q * p.P);
     cs.tok[i] = __ldcg(&p.st.tok[g]);
-    cs.bud[i] = p.st.budget[g];
+    cs.bud[i] = __ldcg(&p.st.budget[g]);
     cs.row[i] = ident ? b0 * p.P + i : __ldcg(&p.row_of[b0 * p.P + i]);
     if (diag) {
       cs.cand[i] = __ldcg(&p.st.cand[g]);
