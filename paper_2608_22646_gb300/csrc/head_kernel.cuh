@@ -429,8 +429,8 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
   // that does (the masked-row count, the gathered rows, the partial buffer,
   // the commit state) is touched only after grid_dependency_wait().  A
   // single-kernel step reads nothing the previous step writes before its
-  // partials, so only its epilogue and its commit wait (and, with wait_rows,
-  // whoever reads the caller's rows).
+  // partials, so only its epilogue and its commit wait (with wait_rows, every
+  // role: no bounded wait of one for another may include the kernel before).
   // When most steps go to the pair kernel, copies started before M is known
   // would mostly be wasted, so the launch asks for none.
   const int n_pre = p.prefetch ? min(p.n_stages, pl.n_tiles * KB) : 0;
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       // ---------------------------------------------------- MMA issuer --
-      if (!p.fused) grid_dependency_wait();
+      if (!p.fused || p.wait_rows) grid_dependency_wait();
       const int M = rows_to_decode(p.d_M, p.fused, p.M_fixed, p.max_M);
       const int n_chunks = (M + kChunkN - 1) / kChunkN;
       Ring ra, rb, racc;
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
     __syncwarp();
   } else {
     // --------------------------------------------------------- epilogue --
-    if (!p.fused) grid_dependency_wait();
+    if (!p.fused || p.wait_rows) grid_dependency_wait();
     const int M = rows_to_decode(p.d_M, p.fused, p.M_fixed, p.max_M);
     const int n_chunks = (M + kChunkN - 1) / kChunkN;
     if (!p.fused && threadIdx.x == 64 && cta == 0 && *p.d_M <= p.max_M) *p.m_hist_slot = M;
@@ -617,7 +617,6 @@ __global__ void __launch_bounds__(kHeadThreads, 1)
     if constexpr (kNorm) {
       __shared__ float s_scale[kChunkN];
       if (p.fused) {
-        if (p.wait_rows) grid_dependency_wait();
         epilogue_row_scales<4>(p.hid, M, p.H, p.norm_eps, s_scale, ew, lane);
         scale = s_scale;
       }

@@ -236,6 +236,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *sm.tmem_slot;
+  // Every role: the bounded waits of one for another must not include the kernel
+  // before this one, however long that takes.
+  if (p.wait_rows) grid_dependency_wait();
 
   bool buffers_free = false;  // thread 0: see fused_step_commit
   if (warp == 0) {
@@ -249,7 +252,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     Ring r;
     int issued = 0;
     bool ok = true, decided = !spec;
-    if (p.wait_rows) grid_dependency_wait();
     // Rows copied from the host on the context's side stream: wait (bounded)
     // for that copy's sequence word before the first row load.
     if (leader && p.stage_word &&
@@ -383,7 +385,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
       // group accumulates.  Nothing here depends on an earlier kernel, so the
       // accumulators are drained as in a step without the norm.
       __shared__ float s_scale[kRowsM];
-      if (p.wait_rows) grid_dependency_wait();
       epilogue_row_scales<kRowsEpiWarps>(p.hid, M, p.H, p.norm_eps, s_scale, warp - 2, lane);
       if (row < M) rs = kLog2e * s_scale[row];
     }
