@@ -35,22 +35,22 @@
  * LM head puts the rows in the MMA's A operand and 256 vocabulary rows in N (up
  * to 128 rows; CAI_ROWS_HEAD=0 uses the swapped-operand kernel instead, W in A
  * and the rows in N).  Otherwise a step is gather, LM head, merge + commit.  The
- * LM head is the CTA-pair kernel (tcgen05 cta_group::2), which picks its orientation per step from
- * the masked-row count M: the rows as MMA N in row tiles of equal width (a
- * multiple of 32) while that width is at most a limit that grows with H (224
- * from H = 3072 on), else as MMA M in 256-row tiles.  A kernel that merges each row's per-tile partials follows it only
- * in contexts where some step size leaves more than one partial per pair and
- * CTA to merge.  CAI_PAIR_SWAP=0 keeps the pair kernel unswapped and moves
- * the steps below 32 rows to the single-CTA swapped-operand kernel (launched
- * on every step, returning at once on the others); CAI_PAIR_SWAP_MAX_N=n sets
- * the widest swapped tile; CAI_PAIR=0 runs every step on the single-CTA
- * kernel; CAI_PAIR_MIN_M=n sets the smallest step of the pair kernel (all
- * read at cai_init; CAI_NVTX=1 wraps every step call in an NVTX range).
- * cai_init_rmsnorm and CAI_DIAGNOSTICS
- * add one small kernel each to a single-kernel step.  The batch runs
- * blocks and steps in lockstep; sequences exit independently (Algorithm 1,
- * per sequence) and contribute no rows afterwards.  A context is not thread
- * safe; use one context per host thread.
+ * LM head is the CTA-pair kernel (tcgen05 cta_group::2), which picks its
+ * orientation per step from the masked-row count M: the rows as MMA N in row
+ * tiles of equal width (a multiple of 32) while that width is at most a limit
+ * that grows with H (cai_pair_swap_limit), else as MMA M in 256-row tiles.  A
+ * kernel that merges each row's per-tile partials follows it only in contexts
+ * where some step size leaves more than one partial per pair and CTA to merge.
+ * CAI_PAIR_SWAP=0 keeps the pair kernel unswapped and moves the steps below 32
+ * rows to the single-CTA swapped-operand kernel (launched on every step,
+ * returning at once on the others); CAI_PAIR_SWAP_MAX_N=n sets the widest
+ * swapped tile; CAI_PAIR=0 runs every step on the single-CTA kernel;
+ * CAI_PAIR_MIN_M=n sets the smallest step of the pair kernel (all read at
+ * cai_init; CAI_NVTX=1 wraps every step call in an NVTX range).
+ * CAI_DIAGNOSTICS adds one small kernel to a step.  The batch runs blocks and
+ * steps in lockstep; sequences exit independently (Algorithm 1, per sequence)
+ * and contribute no rows afterwards.  A context is not thread safe; use one
+ * context per host thread.
  *
  * Status.  Every int-returning call returns CAI_OK (0) or a negative CAI_ERR_*
  * code; no C++ exception crosses the ABI.  After CAI_ERR_CUDA or
@@ -236,8 +236,8 @@ int cai_init(const cai_config* cfg, const void* W, void* stream, cai_ctx** out);
  * call only); eps >= 0.  The weight is folded into the library's packed copies
  * of W (W[v,k] g[k], rounded to bf16 once); 1 / sqrt(mean h^2 + eps) is
  * computed per row in fp32 from the bf16 row and scales the row's logits in
- * fp32 before the softmax.  Single-kernel steps add one small kernel per step
- * for the row scales; multi-kernel steps compute them in the gather.
+ * fp32 before the softmax.  The LM-head kernel of a single-kernel step computes
+ * the row scales itself, the gather those of a multi-kernel step.
  * Errors: as cai_init, and CAI_ERR_ARG for a NULL or misaligned norm_weight or
  * a negative or non-finite eps.
  */

@@ -38,10 +38,10 @@ std::atomic<int> g_head_grid_limit{0};
 // producer may start its dependents early); only the first stages of the weight
 // stream ahead of that.  Measured, microseconds for a whole block of 8 to 12
 // steps, back to back, single- against multi-kernel: 96 rows, 4096 x 126464
-// 1224 against 1264, 1024 x 4096 152 against 178; 99 rows, 1024 x 50003 255
-// against 271, 256 x 16384 193 against 215; 128 rows, 4096 x 126464 1242 against
-// 1271, 3584 x 152064 1297 against 1306, 2048 x 50003 391 against 394, 1024 x
-// 22000 183 against 190.  With a weight of a few MB both are short chains of
+// 1246 against 1284, 1024 x 4096 153 against 180; 99 rows, 1024 x 50003 256
+// against 272, 256 x 16384 195 against 213; 128 rows, 4096 x 126464 1261 against
+// 1287, 3584 x 152064 1311 against 1325, 2048 x 50003 397 against 399, 1024 x
+// 22000 181 against 190.  With a weight of a few MB both are short chains of
 // latencies that differ little, and above 64 rows the multi-kernel step stays:
 // it gets shorter as rows commit.
 constexpr int kFusedMaxRows = 64;       // any weight
@@ -1198,10 +1198,11 @@ int init_impl(const cai_config* cfg_in, const void* W, const void* g, double eps
       return CAI_ERR_CUDA;
     }
   }
-  // All step kernels ask for the same (largest) shared-memory carveout, so the
-  // small gather and merge CTAs can be resident on an SM beside an LM-head
-  // CTA; under programmatic dependent launch they then start, and wait, while
-  // the neighbouring kernel still runs.
+  // All step kernels ask for the same (largest) shared-memory carveout, so that
+  // no SM has to be reconfigured between two of them.  Beside a pair CTA there is
+  // room for a gather CTA in unswapped contexts (H < 384) only, and for a commit
+  // CTA (64000 registers) in none: under programmatic dependent launch those
+  // start as the CTAs of the kernel before them leave their SMs.
   if (cudaFuncSetAttribute(c->head_kernel,
                            cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared) != cudaSuccess ||

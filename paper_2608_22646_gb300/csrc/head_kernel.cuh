@@ -37,10 +37,11 @@
 // ticket, no waiting) merges the partials and applies the commit rule for
 // every sequence (commit.cuh).  A step is then one launch.  Nothing but the
 // commit depends on the previous step: W and the caller's hidden rows are
-// inputs, so under programmatic dependent launch the next step's CTAs start
-// streaming as soon as this step's CTAs leave their SMs, and wait for this
-// step (grid_dependency_wait) only to write their partials (which this
-// step's commit reads) and to commit.  If this step leaves nothing masked,
+// inputs (of more than 64 rows, only the first ring of W is read before the
+// kernel in front of the step has completed: wait_rows), so under programmatic
+// dependent launch the next step's CTAs start streaming as soon as this step's
+// CTAs leave their SMs, and wait for this step (grid_dependency_wait) only to
+// write their partials (which this step's commit reads) and to commit.  If this step leaves nothing masked,
 // the next one learns it from the published step word (CommitParams::pub)
 // while streaming and stops at the next K block.
 //

@@ -29,7 +29,7 @@
 // different row tiles).  Each CTA writes the triples of its half of the
 // vocabulary rows: two partials per pair.  Each CTA loads N / 2 of a tile's
 // rows per K block as one box of exactly that many rows.  A step runs swapped
-// when N is at most swap_max_n (192 by default).
+// when N is at most swap_max_n (by default pair_swap_width(H)).
 //
 // The epilogue of a pair's last tile is not hidden by anything.  With one warp
 // per quarter and a 31-merge transposition per tile it took 6 us at N = 96 and
@@ -93,7 +93,10 @@ namespace cai {
 
 constexpr int kPairEpiWarps = 8;      // two per tensor-memory quarter, half of the columns each
 constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;
-// Registers a thread: a gather CTA (256 threads of at most 56) fits beside a pair CTA.
+// Registers a thread.  No spills at 160, and a block takes the same time at 168
+// (66 to 512 rows, five shapes).  They do not decide what fits beside a pair
+// CTA: with the exchange buffer of swapped contexts its shared memory leaves the
+// SM to nothing else, and a commit CTA (512 threads) would not fit either way.
 constexpr int kPairRegs = 160;
 constexpr int kPairTileRows = 256;    // masked rows per pair tile (MMA M)
 constexpr int kPairTileVocab = 256;   // vocabulary rows per pair tile (MMA N)
@@ -160,7 +163,9 @@ __host__ __device__ inline bool pair_swapped(int M, int swap_max_n) {
 // N = 32 13.7 / 12.6; H = 512 (22000) N = 64 17.4 / 17.5, N = 96 18.5 / 17.6;
 // H = 1024 (50003) N = 96 27.2 / 28.5, N = 160 29.9 / 28.8; H = 2048 (50003)
 // N = 192 48.3 / 46.3, two tiles of 160 57.5 / 66.5; H = 4096 (126464) N = 224
-// 171 / 172, two tiles of 224 271 / 299, N = 256 183 / 182.
+// 171 / 172, two tiles of 224 271 / 299, N = 256 183 / 182.  One limit serves
+// steps of one tile and of several, whose gain is the larger: at H = 2048 the
+// single tiles of 192 lose 2 us so that two tiles of that width win.
 __host__ __device__ inline int pair_swap_width(int H) {
   return H < 384 ? 0 : H < 768 ? 64 : H < 1536 ? 96 : H < 3072 ? 192 : 224;
 }

@@ -24,7 +24,9 @@
 // that no thread loads.  A stage's rows and W complete one barrier and are
 // freed by one commit; with a ring and barriers of their own for the rows a
 // stage took two waits and two commits: 1024 x 22000 11.3 us a step, now 10.0;
-// 2048 x 50003 30.0, now 27.1; 4096 x 126464 with 128 rows 141.8, now 134.2.
+// 2048 x 50003 30.0, now 27.1; 4096 x 126464 with 128 rows 141.8, now 134.2
+// (the figures of this file at 65 to 128 rows: steps back to back without the
+// wait for their rows, HeadParams::wait_rows, which adds 4 to 12 us to each).
 //
 // Work split: as lm_head_softmax_kernel, V in units of 8 rows over the CTAs;
 // a CTA's rows form equal groups of at most 256 vocabulary rows (RowsPlan),
@@ -382,8 +384,8 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
     float rs = kLog2e;
     if constexpr (kNorm) {
       // The final RMSNorm's row scales, from the step's rows while the first
-      // group accumulates.  Nothing here depends on an earlier kernel, so the
-      // accumulators are drained as in a step without the norm.
+      // group accumulates.  Nothing here waits for an earlier kernel (with
+      // wait_rows every role has, above), so the accumulators are drained as in a step without the norm.
       __shared__ float s_scale[kRowsM];
       epilogue_row_scales<kRowsEpiWarps>(p.hid, M, p.H, p.norm_eps, s_scale, warp - 2, lane);
       if (row < M) rs = kLog2e * s_scale[row];

@@ -365,13 +365,14 @@ __global__ void __launch_bounds__(kCommitThreads) merge_commit_kernel(const Comm
     M = p.t == 0 ? p.B * p.P : __ldcg(p.d_M);
     commit_load(p, blockIdx.x, 1, cs);
   }
-  // With prefetch_state the CTA is resident long before the partials are
-  // there: it makes a first pass over whatever the buffers hold, writing
-  // nothing, so that the code (which the step's weight stream has pushed out
-  // of the caches) is there when the second, real pass has to be quick.  From
-  // the partials to the published step: 12.7 -> 7.7 us (4096 x 126464, two
-  // sequences of 33 rows); a step 163 -> 159 us with the LM head's earlier
-  // set-up.
+  // With prefetch_state the CTA starts when the first pair CTAs have left their
+  // SMs (none fits beside one), while the last pairs end and the grid completes,
+  // a few microseconds.  In them it makes a first pass over whatever the buffers
+  // hold, writing nothing, so that the code (which the step's weight stream has
+  // pushed out of the caches) is there when the second, real pass has to be
+  // quick.  Blocks of eight steps without and with it: 66 rows, 4096 x 126464
+  // 1269.5 -> 1265.2 us, 256 rows, 1024 x 22000 197.4 -> 192.6 us; within the
+  // noise at 352 and 512 rows.
 #pragma unroll 1
   for (int pass = p.prefetch_state ? 0 : 1; pass < 2; ++pass) {
     const bool real = pass == 1;
